@@ -36,9 +36,9 @@ __device__ __forceinline__ bool load_input(const TraceArgs& A, int64_t i, Ray<R>
   n->x = static_cast<const R*>(A.in_x)[i];
   n->y = static_cast<const R*>(A.in_y)[i];
   n->z = static_cast<const R*>(A.in_z)[i];
-  n->dx = vx / sp;
-  n->dy = vy / sp;
-  n->dz = vz / sp;
+  n->dx = Mth<R>::div(vx, sp);
+  n->dy = Mth<R>::div(vy, sp);
+  n->dz = Mth<R>::div(vz, sp);
   n->speed = sp;
   n->t.set(A.in_t[i]);
   n->w = static_cast<const R*>(A.in_w)[i];
@@ -65,7 +65,7 @@ __device__ __forceinline__ R step_segments(const TraceArgs& A, const SampleP<R>&
   st.ns = assembly_segs<R, NS>(S, L.n, st.seg);
 #pragma unroll
   for (int j = 0; j < NS; ++j)
-    st.mu[j] = S.s[j].n100 * (S.s[j].sig_s + S.s[j].sab2200 / L.n.speed);
+    st.mu[j] = S.s[j].n100 * (S.s[j].sig_s + M::div(S.s[j].sab2200, L.n.speed));
   R tau = R(0), len_tot = R(0), lg = R(0);
 #pragma unroll
   for (int k = 0; k < 2 * NS; ++k) {
@@ -151,7 +151,7 @@ __device__ __forceinline__ bool step_scatter(const TraceArgs& A, const SampleP<R
   L.n.x += s_pt * L.n.dx;
   L.n.y += s_pt * L.n.dy;
   L.n.z += s_pt * L.n.dz;
-  L.n.t.add(s_pt / L.n.speed);
+  L.n.t.add(M::div(s_pt, L.n.speed));
   const int kk = (sc.nk == 2 && !(u_k * sc.ksig_sum < sc.ksig0)) ? 1 : 0;
   Scatter<R> out;
   const bool ok = scatter_kernel<R, KS>(S, sc, kk, rng, L.o, &L.n, &out, &pol.err);

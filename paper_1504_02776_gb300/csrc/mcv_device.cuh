@@ -11,6 +11,7 @@
 #include <math_constants.h>
 
 #include "mcv_params.h"
+#include "mcv_soft64.cuh"
 
 namespace mcv {
 
@@ -20,6 +21,7 @@ struct Mth;
 
 template <>
 struct Mth<float> {
+  static __device__ __forceinline__ float div(float a, float b) { return a / b; }
   static __device__ __forceinline__ float sqrt(float x) { return sqrtf(x); }
   // exp and log from the hardware approximations (a few ulp; subnormals kept, so a tiny
   // table value or weight is not flushed to zero)
@@ -52,21 +54,26 @@ struct Mth<float> {
 
 template <>
 struct Mth<double> {
-  static __device__ __forceinline__ double sqrt(double x) { return ::sqrt(x); }
-  static __device__ __forceinline__ double exp(double x) { return ::exp(x); }
-  static __device__ __forceinline__ double log(double x) { return ::log(x); }
+  // on the integer pipes (mcv_soft64.cuh): division and square root with the FP64 pipe's
+  // results, the elementary functions at least as accurate as the library's
+  static __device__ __forceinline__ double div(double a, double b) { return soft64::div(a, b); }
+  static __device__ __forceinline__ double sqrt(double x) { return soft64::sqrt(x); }
+  static __device__ __forceinline__ double exp(double x) { return soft64::exp(x); }
+  static __device__ __forceinline__ double log(double x) { return soft64::log(x); }
   static __device__ __forceinline__ double log1p(double x) { return ::log1p(x); }
   static __device__ __forceinline__ double expm1(double x) { return ::expm1(x); }
-  static __device__ __forceinline__ double tan(double x) { return ::tan(x); }
+  static __device__ __forceinline__ double tan(double x) { return soft64::tan(x); }
   static __device__ __forceinline__ double atan2(double y, double x) { return ::atan2(y, x); }
   static __device__ __forceinline__ double floor(double x) { return ::floor(x); }
   static __device__ __forceinline__ double fabs(double x) { return ::fabs(x); }
   static __device__ __forceinline__ double fmin(double a, double b) { return ::fmin(a, b); }
   static __device__ __forceinline__ double fmax(double a, double b) { return ::fmax(a, b); }
   static __device__ __forceinline__ double hypot(double a, double b) { return ::hypot(a, b); }
-  // the FP64 mode evaluates sin and cos of (2 pi) u as written
+  // sin and cos of the double (2 pi) u
   static __device__ __forceinline__ void sincos2pi(double u, double* s, double* c) {
-    ::sincos(2.0 * kPi * u, s, c);
+    const double2 sc = soft64::sincos2pi(u);
+    *s = sc.x;
+    *c = sc.y;
   }
   static __device__ __forceinline__ double inf() { return CUDART_INF; }
   static __device__ __forceinline__ double cos_(double x) { return ::cos(x); }
@@ -255,9 +262,9 @@ __device__ __forceinline__ void beam_divergence(const BeamP<double>& B,
   const double ax = B.div * (rr * c), ay = B.div * (rr * s);
   const double tx = M::tan(ax), ty = M::tan(ay);
   const double norm = M::sqrt(tx * tx + ty * ty + 1.0);
-  n->dx = tx / norm;
-  n->dy = ty / norm;
-  n->dz = 1.0 / norm;
+  n->dx = M::div(tx, norm);
+  n->dy = M::div(ty, norm);
+  n->dz = M::div(1.0, norm);
   *aux = 0.0;
 }
 
@@ -272,8 +279,8 @@ __device__ __forceinline__ bool beam_energy(const BeamP<double>& B,
   const double zE = M::sqrt(-2.0 * M::log(u0)) * c;
   const double E = B.ei * (1.0 + B.rel * zE);
   if (!(E > 0.0)) return false;
-  n->speed = M::sqrt(E / kMeVPerV2);
-  n->t.set((B.l1 - B.z0) / (n->speed * n->dz));
+  n->speed = M::sqrt(M::div(E, kMeVPerV2));
+  n->t.set(M::div(B.l1 - B.z0, n->speed * n->dz));
   return true;
 }
 
@@ -361,11 +368,11 @@ __device__ __forceinline__ bool cyl_span(R rad, R x, R z, R dx, R dz, R* s1, R* 
     }
     return false;
   }
-  const R tc = -(x * dx + z * dz) / a;
+  const R tc = M::div(-(x * dx + z * dz), a);
   const R cr = x * dz - z * dx;
-  const R g = rad * rad - cr * cr / a;
+  const R g = rad * rad - M::div(cr * cr, a);
   if (!(g > R(0))) return false;
-  const R half = M::sqrt(g / a);
+  const R half = M::sqrt(M::div(g, a));
   *s1 = tc - half;
   *s2 = tc + half;
   return true;
@@ -383,7 +390,7 @@ __device__ __forceinline__ bool slab_span(R half, R p, R dp, R* s1, R* s2) {
     }
     return false;
   }
-  const R a = (-half - p) / dp, b = (half - p) / dp;
+  const R a = M::div(-half - p, dp), b = M::div(half - p, dp);
   *s1 = M::fmin(a, b);
   *s2 = M::fmax(a, b);
   return true;
@@ -521,7 +528,7 @@ __device__ __forceinline__ void turn(R c, R s, R u, R* dx, R* dy, R* dz) {
     e1y = -z;
     e1z = y;
   }
-  const R inv = R(1) / M::sqrt(e1x * e1x + e1y * e1y + e1z * e1z);
+  const R inv = M::div(R(1), M::sqrt(e1x * e1x + e1y * e1y + e1z * e1z));
   e1x *= inv;
   e1y *= inv;
   e1z *= inv;
@@ -571,7 +578,7 @@ __device__ __forceinline__ bool kernel_sqe(const SampleP<R>& S, const Rng& rng, 
   // Ef = Ei - E; when the range ends at Ei it is the sampled offset from that end
   const R Ef = (e_hi == Ei) ? (R(1) - u0) * dE : Ei - E;
   if (!(Ef > R(0))) return false;
-  const R speed_f = M::sqrt(Ef / (R)kMeVPerV2);
+  const R speed_f = M::sqrt(M::div(Ef, (R)kMeVPerV2));
   const R kf = (R)kKPerV * speed_f;
   const R q_lo = M::fabs(ki - kf);
   const R q_hi = M::fmin(ki + kf, (R)S.q_max);
@@ -581,13 +588,13 @@ __device__ __forceinline__ bool kernel_sqe(const SampleP<R>& S, const Rng& rng, 
   // cos and sin of the scattering angle from 1 -/+ cos, each a product whose small factor
   // is the sampled offset from an end of the Q range (no cancellation near 0 or pi)
   const R den = R(2) * ki * kf;
-  const R one_m = (u1 * dQ) * (Q + q_lo) / den;
+  const R one_m = M::div((u1 * dQ) * (Q + q_lo), den);
   const R top = (q_hi == ki + kf) ? (R(1) - u1) * dQ : (ki + kf) - Q;
-  const R one_p = top * (ki + kf + Q) / den;
+  const R one_p = M::div(top * (ki + kf + Q), den);
   R c2t = (one_m <= one_p) ? R(1) - one_m : one_p - R(1);
   c2t = M::fmin(R(1), M::fmax(R(-1), c2t));
   const R s2t = M::sqrt(M::fmax(R(0), one_m * one_p));
-  const R fq = M::floor(Q / (R)S.dq), fe = M::floor((E - (R)S.e_min) / (R)S.de);
+  const R fq = M::floor(M::div(Q, (R)S.dq)), fe = M::floor(M::div(E - (R)S.e_min, (R)S.de));
   if (!(fq >= R(0) && fq < (R)S.nq && fe >= R(0) && fe < (R)S.ne)) return false;
   const int entry = (int)fq * S.ne + (int)fe;
   if (entry < 0 || entry >= S.nq * S.ne) {
@@ -598,7 +605,7 @@ __device__ __forceinline__ bool kernel_sqe(const SampleP<R>& S, const Rng& rng, 
   const R u2 = rng.template first<R>(o, 2);
   turn<R>(c2t, s2t, u2, &n->dx, &n->dy, &n->dz);
   n->speed = speed_f;
-  sc->rest = Q * dE * dQ / (R(2) * ki * ki);
+  sc->rest = M::div(Q * dE * dQ, R(2) * ki * ki);
   sc->factor = Sv * sc->rest;
   sc->s_value = Sv;
   sc->entry = entry;
@@ -653,7 +660,7 @@ __device__ __forceinline__ bool kernel_phonon(const SampleP<R>& S, const Rng& rn
     n->dx = dx;
     n->dy = dy;
     n->dz = dz;
-    sc->rest = M::exp(-S.ph_cw * q * q) / S.ph_p0;
+    sc->rest = M::div(M::exp(-S.ph_cw * q * q), S.ph_p0);
     sc->factor = sc->rest;
     sc->q = q;
     sc->e = R(0);
@@ -661,7 +668,7 @@ __device__ __forceinline__ bool kernel_phonon(const SampleP<R>& S, const Rng& rn
   }
   const bool one = u0 < S.ph_p01;
   const R p_ch = one ? S.ph_p1 : S.ph_p2;
-  const R ue = (u0 - (one ? S.ph_p0 : S.ph_p01)) / p_ch;
+  const R ue = M::div(u0 - (one ? S.ph_p0 : S.ph_p01), p_ch);
   // one search for both channels (the lanes of a warp pick either), from A_1 or from B
   const int k = draw_mass<R>(one ? S.ph_cdf1 : S.ph_cdfb, one ? 2 * S.ph_J + 1 : S.ph_M, ue);
   const int i = k - (one ? S.ph_J : S.ph_N * S.ph_J);
@@ -669,15 +676,15 @@ __device__ __forceinline__ bool kernel_phonon(const SampleP<R>& S, const Rng& rn
   const R E = ((R)i + (u1 - R(0.5))) * S.ph_de;
   const R Ef = Ei - E;
   if (!(Ef > R(0))) return false;
-  const R speed_f = M::sqrt(Ef / (R)kMeVPerV2);
+  const R speed_f = M::sqrt(M::div(Ef, (R)kMeVPerV2));
   const R kf = (R)kKPerV * speed_f;
   const R q_lo = M::fabs(ki - kf), q_hi = ki + kf;
   const R dQ = q_hi - q_lo;
   const R Q = q_lo + u2 * dQ;
   // scattering angle from 1 -/+ cos as products of the offsets from the ends of the range
   const R den = R(2) * ki * kf;
-  const R one_m = (u2 * dQ) * (Q + q_lo) / den;
-  const R one_p = ((R(1) - u2) * dQ) * (ki + kf + Q) / den;
+  const R one_m = M::div((u2 * dQ) * (Q + q_lo), den);
+  const R one_p = M::div(((R(1) - u2) * dQ) * (ki + kf + Q), den);
   R c2t = (one_m <= one_p) ? R(1) - one_m : one_p - R(1);
   c2t = M::fmin(R(1), M::fmax(R(-1), c2t));
   const R s2t = M::sqrt(M::fmax(R(0), one_m * one_p));
@@ -692,13 +699,13 @@ __device__ __forceinline__ bool kernel_phonon(const SampleP<R>& S, const Rng& rn
     for (int k = 2; k <= S.ph_N; ++k) {
       pw *= w2;
       fact *= (R)k;
-      sum += pw / fact * __ldg(S.ph_an + (int64_t)(k - 2) * S.ph_M + g);
+      sum += M::div(pw, fact) * __ldg(S.ph_an + (int64_t)(k - 2) * S.ph_M + g);
     }
-    ratio = M::exp(-w2) * sum / mass;
+    ratio = M::div(M::exp(-w2) * sum, mass);
   }
   turn<R>(c2t, s2t, u3, &n->dx, &n->dy, &n->dz);
   n->speed = speed_f;
-  sc->rest = ratio * Q * dQ / (R(2) * ki * ki) / p_ch;
+  sc->rest = M::div(M::div(ratio * Q * dQ, R(2) * ki * ki), p_ch);
   sc->factor = sc->rest;
   sc->q = Q;
   sc->e = E;
@@ -719,7 +726,7 @@ __device__ __forceinline__ bool kernel_bragg(const SampleP<R>& S, R sig_k, const
                                              int o, Ray<R>* n, Scatter<R>* sc) {
   using M = Mth<R>;
   const R ki = (R)kKPerV * n->speed;
-  const R lam = R(2.0 * kPi) / ki;
+  const R lam = M::div(R(2.0 * kPi), ki);
   int lo = 0, hi = S.n_refl;  // allowed: the reflections with lam < 2 d
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
@@ -742,11 +749,11 @@ __device__ __forceinline__ bool kernel_bragg(const SampleP<R>& S, R sig_k, const
     else lo = mid + 1;
   }
   const int pick = lo;
-  const R s = lam / (R(2) * __ldg(S.refl_d + pick));
+  const R s = M::div(lam, R(2) * __ldg(S.refl_d + pick));
   const R c2t = R(1) - R(2) * s * s;
   const R s2t = R(2) * s * M::sqrt((R(1) - s) * (R(1) + s));
   turn<R>(c2t, s2t, u1, &n->dx, &n->dy, &n->dz);
-  sc->rest = total / sig_k;
+  sc->rest = M::div(total, sig_k);
   sc->factor = sc->rest;
   sc->s_value = R(1);
   sc->entry = -1;
@@ -816,15 +823,15 @@ __device__ __forceinline__ void eig3_branch(const R D[6], int b, R* lam, R* ex, 
     return;
   }
   // Cardano estimates
-  const R q = (a00 + a11 + a22) / R(3);
+  const R q = M::div(a00 + a11 + a22, R(3));
   const R p2 = (a00 - q) * (a00 - q) + (a11 - q) * (a11 - q) + (a22 - q) * (a22 - q) + R(2) * p1;
-  const R p = M::sqrt(p2 / R(6));
-  const R b00 = (a00 - q) / p, b11 = (a11 - q) / p, b22 = (a22 - q) / p;
-  const R b01 = a01 / p, b02 = a02 / p, b12 = a12 / p;
+  const R p = M::sqrt(M::div(p2, R(6)));
+  const R b00 = M::div(a00 - q, p), b11 = M::div(a11 - q, p), b22 = M::div(a22 - q, p);
+  const R b01 = M::div(a01, p), b02 = M::div(a02, p), b12 = M::div(a12, p);
   R r = R(0.5) * (b00 * (b11 * b22 - b12 * b12) - b01 * (b01 * b22 - b12 * b02) +
                   b02 * (b01 * b12 - b11 * b02));
   r = M::fmin(R(1), M::fmax(R(-1), r));
-  const R phi = M::acos_(r) / R(3);
+  const R phi = M::div(M::acos_(r), R(3));
   const R l2 = q + R(2) * p * M::cos_(phi);
   const R l0 = q + R(2) * p * M::cos_(phi + R(2) * (R)kPi / R(3));
   const R l1 = R(3) * q - l0 - l2;
@@ -850,7 +857,7 @@ __device__ __forceinline__ void eig3_branch(const R D[6], int b, R* lam, R* ex, 
     }
   }
   if (nb > R(0)) {
-    const R inv = R(1) / M::sqrt(nb);
+    const R inv = M::div(R(1), M::sqrt(nb));
     gx = gx * inv;
     gy = gy * inv;
     gz = gz * inv;
@@ -880,7 +887,7 @@ __device__ __forceinline__ void eig3_branch(const R D[6], int b, R* lam, R* ex, 
     uy = -gx;
     uz = R(0);
   }
-  const R un = R(1) / M::sqrt(ux * ux + uy * uy + uz * uz);
+  const R un = M::div(R(1), M::sqrt(ux * ux + uy * uy + uz * uz));
   ux = ux * un;
   uy = uy * un;
   uz = uz * un;
@@ -919,8 +926,8 @@ __device__ __forceinline__ void eig3_branch(const R D[6], int b, R* lam, R* ex, 
   }
   const R cn = M::hypot(cu, cw);
   if (cn > R(0)) {
-    cu = cu / cn;
-    cw = cw / cn;
+    cu = M::div(cu, cn);
+    cw = M::div(cw, cn);
   } else {
     cu = R(1);
     cw = R(0);
@@ -956,7 +963,7 @@ __device__ __forceinline__ BvkPoint<R> bvk_point(const SampleP<R>& S, R c, R s, 
                                                   R dix, R diy, R diz, R dfx, R dfy, R dfz,
                                                   R Ef, int b, int sg) {
   BvkPoint<R> P;
-  const R kf = (R)kKPerV * Mth<R>::sqrt(Ef / (R)kMeVPerV2);
+  const R kf = (R)kKPerV * Mth<R>::sqrt(Mth<R>::div(Ef, (R)kMeVPerV2));
   const R Qx = dix * ki - dfx * kf, Qy = diy * ki - dfy * kf, Qz = diz * ki - dfz * kf;
   to_crystal<R>(c, s, Qx, Qy, Qz, &P.qx, &P.qy, &P.qz);
   R D[6];
@@ -1024,8 +1031,8 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
   if (!(P.hw >= R(1e-3))) return false;
   const R ex = P.ex, ey = P.ey, ez = P.ez;
   // d hw / d Ef through Q(Ef) (Hellmann-Feynman: d lambda = e^T dD e)
-  const R kf = (R)kKPerV * M::sqrt(Ef / (R)kMeVPerV2);
-  const R dkf = kf / (R(2) * Ef);
+  const R kf = (R)kKPerV * M::sqrt(M::div(Ef, (R)kMeVPerV2));
+  const R dkf = M::div(kf, R(2) * Ef);
   R dqx, dqy, dqz;
   to_crystal<R>(crot, srot, dfx, dfy, dfz, &dqx, &dqy, &dqz);
   dqx *= -dkf;
@@ -1041,15 +1048,15 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
     const R dqd = S.bvk_ah * (dqx * v[0] + dqy * v[1] + dqz * v[2]);
     dlam += R(2) * M::sin_(qd) * dqd * ed * ed * R(0.5);
   }
-  const R dhw = S.bvk_hwu * dlam / (R(2) * M::sqrt(P.lam));
+  const R dhw = M::div(S.bvk_hwu * dlam, R(2) * M::sqrt(P.lam));
   const R gp = R(-1) - (R)sg * dhw;
-  const R nB = R(1) / M::expm1(P.hw / S.bvk_kT);
+  const R nB = M::div(R(1), M::expm1(M::div(P.hw, S.bvk_kT)));
   const R Ns = sg > 0 ? nB + R(1) : nB;
   const R qe = P.qx * ex + P.qy * ey + P.qz * ez;
   const R Q2 = P.qx * P.qx + P.qy * P.qy + P.qz * P.qz;
-  const R dw = M::exp(-Q2 * S.bvk_msd / R(3));
-  const R Rb = S.bvk_hb2m * qe * qe / P.hw;
-  sc->rest = R(6) * (R)nroots * (kf / ki) * dw * Rb * Ns / M::fabs(gp);
+  const R dw = M::exp(M::div(-Q2 * S.bvk_msd, R(3)));
+  const R Rb = M::div(S.bvk_hb2m * qe * qe, P.hw);
+  sc->rest = M::div(R(6) * (R)nroots * M::div(kf, ki) * dw * Rb * Ns, M::fabs(gp));
   sc->factor = sc->rest;
   sc->s_value = R(1);
   sc->entry = -1;
@@ -1058,7 +1065,7 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
   n->dx = dfx;
   n->dy = dfy;
   n->dz = dfz;
-  n->speed = M::sqrt(Ef / (R)kMeVPerV2);
+  n->speed = M::sqrt(M::div(Ef, (R)kMeVPerV2));
   return true;
 }
 
@@ -1079,7 +1086,7 @@ __device__ __forceinline__ DispPoint<R> disp_point(const SampleP<R>& S, R c, R s
                                                     R Ef) {
   using M = Mth<R>;
   DispPoint<R> P;
-  const R kf = (R)kKPerV * M::sqrt(Ef / (R)kMeVPerV2);
+  const R kf = (R)kKPerV * M::sqrt(M::div(Ef, (R)kMeVPerV2));
   const R Qx = dix * ki - dfx * kf, Qy = diy * ki - dfy * kf, Qz = diz * ki - dfz * kf;
   R qx, qy, qz;
   to_crystal<R>(c, s, Qx, Qy, Qz, &qx, &qy, &qz);
@@ -1142,17 +1149,17 @@ __device__ __forceinline__ bool kernel_disp(const SampleP<R>& S, R crot, R srot,
   const DispPoint<R> P = disp_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy,
                                        dfz, Ef);
   if (!(P.E > R(0))) return false;
-  const R kf = (R)kKPerV * M::sqrt(Ef / (R)kMeVPerV2);
+  const R kf = (R)kKPerV * M::sqrt(M::div(Ef, (R)kMeVPerV2));
   R dqx, dqy, dqz;
   to_crystal<R>(crot, srot, dfx, dfy, dfz, &dqx, &dqy, &dqz);
-  const R sc_q = -kf / (R(2) * Ef);
+  const R sc_q = M::div(-kf, R(2) * Ef);
   dqx *= sc_q;
   dqz *= sc_q;
   const R ac = S.disp_amp * S.disp_c;
-  const R gx = ac * P.sa * P.ca * P.cb * P.cb / P.root;
-  const R gz = ac * P.ca * P.ca * P.sb * P.cb / P.root;
+  const R gx = M::div(ac * P.sa * P.ca * P.cb * P.cb, P.root);
+  const R gz = M::div(ac * P.ca * P.ca * P.sb * P.cb, P.root);
   const R gp = R(-1) - (gx * dqx + gz * dqz);
-  sc->rest = (R)nroots * (kf / ki) * S.disp_s0 / M::fabs(gp);
+  sc->rest = M::div((R)nroots * M::div(kf, ki) * S.disp_s0, M::fabs(gp));
   sc->factor = sc->rest;
   sc->s_value = R(1);
   sc->entry = -1;
@@ -1161,7 +1168,7 @@ __device__ __forceinline__ bool kernel_disp(const SampleP<R>& S, R crot, R srot,
   n->dx = dfx;
   n->dy = dfy;
   n->dz = dfz;
-  n->speed = M::sqrt(Ef / (R)kMeVPerV2);
+  n->speed = M::sqrt(M::div(Ef, (R)kMeVPerV2));
   return true;
 }
 
@@ -1195,11 +1202,11 @@ __device__ __forceinline__ bool tube_span(R Rad, R ux, R uz, R rt, const Ray<R>&
   const R o_tan = n.x * uz - n.z * ux;
   const R d_rad = n.dx * ux + n.dz * uz;
   const R d_tan = n.dx * uz - n.dz * ux;
-  const R tc = -(o_rad * d_rad + o_tan * d_tan) / a;
+  const R tc = Mth<R>::div(-(o_rad * d_rad + o_tan * d_tan), a);
   const R cr = o_rad * d_tan - o_tan * d_rad;
-  const R g = rt * rt - cr * cr / a;
+  const R g = rt * rt - Mth<R>::div(cr * cr, a);
   if (!(g > R(0))) return false;
-  const R half = Mth<R>::sqrt(g / a);
+  const R half = Mth<R>::sqrt(Mth<R>::div(g, a));
   *s1 = tc - half;
   *s2 = tc + half;
   return true;
@@ -1211,7 +1218,7 @@ template <typename R>
 __device__ __forceinline__ int64_t tof_bin(const TofWin& W, const Tof<R>& tof);
 template <>
 __device__ __forceinline__ int64_t tof_bin<double>(const TofWin& W, const Tof<double>& tof) {
-  const double fb = ::floor((tof.v - W.tof_min) / W.dt);
+  const double fb = ::floor(soft64::div(tof.v - W.tof_min, W.dt));
   if (!(fb >= 0.0 && fb < (double)W.n_tof)) return -1;
   return (int64_t)fb;
 }
@@ -1240,12 +1247,12 @@ __device__ __forceinline__ Hit<R> detect_surface(const DetP<R>& D, const TofWin&
   if (yh < -half || yh >= half) return h;
   const R xh = n.x + s * n.dx, zh = n.z + s * n.dz;
   const R phi = M::atan2(xh, zh);
-  int ip = (int)M::floor((phi + (R)kPi) / (R)(2.0 * kPi) * (R)D.n_phi);
+  int ip = (int)M::floor(M::div(phi + (R)kPi, (R)(2.0 * kPi)) * (R)D.n_phi);
   ip = min(max(ip, 0), D.n_phi - 1);
-  int iy = (int)M::floor((yh + half) / (R)D.height * (R)D.n_y);
+  int iy = (int)M::floor(M::div(yh + half, (R)D.height) * (R)D.n_y);
   iy = min(max(iy, 0), D.n_y - 1);
   h.pixel = ip * D.n_y + iy;
-  h.tof.add(s / n.speed);
+  h.tof.add(M::div(s, n.speed));
   h.w_det = n.w;
   h.pabs = R(1);
   const int64_t tb = tof_bin<R>(W, h.tof);
@@ -1296,9 +1303,9 @@ __device__ __forceinline__ bool tubes_locate(const DetP<R>& D, const Ray<R>& n, 
   const int tpp = D.tubes_per_pack;
   const R period = (R)D.period, pitch = (R)D.pitch;
   const R arc = (M::atan2(Px, Pz) - (R)D.phi0) * Rad;
-  const R p = M::floor(arc / period);
+  const R p = M::floor(M::div(arc, period));
   const R within = arc - p * period;
-  R k = M::floor(within / pitch);
+  R k = M::floor(M::div(within, pitch));
   if (k > (R)(tpp - 1)) k = (R)(tpp - 1);
   // more than one tube outside the rows' arc: no candidate (the range check on the float
   // also keeps its conversion to int in range)
@@ -1344,7 +1351,7 @@ __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W
       ys1 = -M::inf();
       ys2 = M::inf();
     } else {
-      const R a = (y_lo - n.y) / n.dy, b = (y_hi - n.y) / n.dy;
+      const R a = M::div(y_lo - n.y, n.dy), b = M::div(y_hi - n.y, n.dy);
       ys1 = M::fmin(a, b);
       ys2 = M::fmax(a, b);
     }
@@ -1359,16 +1366,16 @@ __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W
   }
   if (best < 0) return h;
   const R L = best_out - best_in;
-  const R mu = (R)D.mu_he_v / n.speed;
+  const R mu = M::div((R)D.mu_he_v, n.speed);
   const R pabs = -M::expm1(-mu * L);
-  const R x = -M::log1p(-u_det * pabs) / mu;
+  const R x = M::div(-M::log1p(-u_det * pabs), mu);
   const R s_abs = best_in + x;
   const R y_abs = n.y + s_abs * n.dy;
-  int j = (int)M::floor((y_abs - y_lo) / (R)D.pix_len);
+  int j = (int)M::floor(M::div(y_abs - y_lo, (R)D.pix_len));
   j = min(max(j, 0), D.pixels_per_tube - 1);
   const int pc = best / tpp, tc = best - pc * tpp;
   h.pixel = ((row_off + pc) * tpp + tc) * D.pixels_per_tube + j;
-  h.tof.add(s_abs / n.speed);
+  h.tof.add(M::div(s_abs, n.speed));
   h.pabs = pabs;
   h.w_det = n.w * pabs;
   const int64_t tb = tof_bin<R>(W, h.tof);

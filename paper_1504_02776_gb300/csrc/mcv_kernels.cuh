@@ -826,7 +826,7 @@ struct Adjoint {
     }
     const ScatP<R>& g = Sof<R>(A).s[A.gs];
     const R w_det = we * h.pabs;
-    const R dabs = cum_dabs - g.n100 * (R(2200) / L.n.speed) * lg;
+    const R dabs = cum_dabs - g.n100 * Mth<R>::div(R(2200), L.n.speed) * lg;
     const R ds = cum_ds - g.n100 * lg;
     acc_abs.add(gb * w_det * dabs);
     acc_s.add(gb * w_det * ds);
@@ -852,9 +852,9 @@ struct Adjoint {
     s[k] = out.s_value;
     e[k] = out.entry;
     const ScatP<R>& g = Sof<R>(A).s[A.gs];
-    cum_dabs -= g.n100 * (R(2200) / speed_in) * lg_pt;
+    cum_dabs -= g.n100 * Mth<R>::div(R(2200), speed_in) * lg_pt;
     cum_ds -= g.n100 * lg_pt;
-    if (j == A.gs) cum_ds += R(1) / g.sig_s;
+    if (j == A.gs) cum_ds += Mth<R>::div(R(1), g.sig_s);
   }
 
   __device__ __forceinline__ void clear(const TraceArgs&, int64_t, int) {}

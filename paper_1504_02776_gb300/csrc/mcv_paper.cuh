@@ -85,7 +85,7 @@ __device__ __forceinline__ int tubes_absorb_multi(const DetP<R>& D, const TofWin
       ys1 = -M::inf();
       ys2 = M::inf();
     } else {
-      const R a = (y_lo - n.y) / n.dy, b = (y_hi - n.y) / n.dy;
+      const R a = M::div(y_lo - n.y, n.dy), b = M::div(y_hi - n.y, n.dy);
       ys1 = M::fmin(a, b);
       ys2 = M::fmax(a, b);
     }
@@ -102,20 +102,20 @@ __device__ __forceinline__ int tubes_absorb_multi(const DetP<R>& D, const TofWin
     s_in[at] = a_in;
     s_out[at] = a_out;
   }
-  const R mu = (R)D.mu_he_v / n.speed;
+  const R mu = M::div((R)D.mu_he_v, n.speed);
   R left = n.w;
   for (int i = 0; i < m; ++i) {
     const R L = s_out[i] - s_in[i];
     const R pabs = -M::expm1(-mu * L);
-    const R x = -M::log1p(-u[i] * pabs) / mu;
+    const R x = M::div(-M::log1p(-u[i] * pabs), mu);
     const R s_abs = s_in[i] + x;
     const R y_abs = n.y + s_abs * n.dy;
-    int j = (int)M::floor((y_abs - y_lo) / (R)D.pix_len);
+    int j = (int)M::floor(M::div(y_abs - y_lo, (R)D.pix_len));
     j = min(max(j, 0), D.pixels_per_tube - 1);
     const int pc = tube[i] / tpp, tc = tube[i] - pc * tpp;
     h[i].pixel = ((row_off + pc) * tpp + tc) * D.pixels_per_tube + j;
     h[i].tof = n.t;
-    h[i].tof.add(s_abs / n.speed);
+    h[i].tof.add(M::div(s_abs, n.speed));
     h[i].pabs = pabs;
     h[i].w_det = left * pabs;
     left = left * (R(1) - pabs);
@@ -215,7 +215,7 @@ __device__ __forceinline__ void paper_propagate_out(const SampleP<R>& S, const S
   for (int k = 0; k < 2 * NS; ++k) {
     if (k < ns) {
       const ScatP<R>& sc = S.s[seg[k].j];
-      tau += sc.n100 * (sc.sig_s + sc.sab2200 / p->n.speed) * (seg[k].b - seg[k].a);
+      tau += sc.n100 * (sc.sig_s + Mth<R>::div(sc.sab2200, p->n.speed)) * (seg[k].b - seg[k].a);
     }
   }
   p->n.w = p->n.w * Mth<R>::exp(-tau);
@@ -230,7 +230,7 @@ __device__ __forceinline__ int paper_interact1(const TraceArgs& A, const SampleP
   using M = Mth<R>;
   const ScatP<R>& sc = S.s[j];
   const R len = b - a;
-  const R mu = sc.n100 * (sc.sig_s + sc.sab2200 / in.n.speed);
+  const R mu = sc.n100 * (sc.sig_s + M::div(sc.sab2200, in.n.speed));
   *tr = in;
   tr->s0 = b;
   tr->n.w = in.n.w * M::exp(-mu * len);
@@ -244,7 +244,7 @@ __device__ __forceinline__ int paper_interact1(const TraceArgs& A, const SampleP
   p.n.x = in.n.x + in.n.dx * s;
   p.n.y = in.n.y + in.n.dy * s;
   p.n.z = in.n.z + in.n.dz * s;
-  p.n.t.add(s / in.n.speed);
+  p.n.t.add(M::div(s, in.n.speed));
   p.n.w = in.n.w * sc.mu_s * len * M::exp(-mu * ell);
   p.s0 = R(0);
   const int kk = (sc.nk == 2 && !(u_k * sc.ksig_sum < sc.ksig0)) ? 1 : 0;
