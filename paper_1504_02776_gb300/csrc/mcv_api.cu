@@ -32,6 +32,13 @@ mcv_status alloc_fail(const std::string& msg) {
 
 bool is_finite(double v) { return std::isfinite(v); }
 
+namespace {
+void no_miss_bounds(mcv::BeamP<double>* B) {
+  B->fx_lo = B->fy_lo = 0;
+  B->fx_hi = B->fy_hi = 0xffffffffu;
+}
+}  // namespace
+
 // ---- descriptions -> device parameter blocks -------------------------------------------
 mcv_status build_beam(const mcv_beam_params* b, mcv::BeamP<double>* B) {
   if (!b) return fail(MCV_EINVAL, "beam parameters are NULL");
@@ -55,8 +62,7 @@ mcv_status build_beam(const mcv_beam_params* b, mcv::BeamP<double>* B) {
   B->t0_hi = (float)B->t0;
   B->t0_lo = (float)(B->t0 - (double)B->t0_hi);
   B->energy_positive = b->ei_rel_sigma * 8.7 < 1.0 ? 1 : 0;
-  B->x_safe = INFINITY;
-  B->y_safe = INFINITY;
+  no_miss_bounds(B);
   return MCV_OK;
 }
 
@@ -289,10 +295,10 @@ mcv_status build_detector(const mcv_detector* d, mcv::DetP<double>* D) {
 // uniforms can give: the sample lies within radius r of the vertical axis and |y| <= hh; a
 // ray from the start plane z = -z0 with divergence angles |a| <= 8.66 div (Box-Muller
 // normals of uniforms >= 2^-54 stay within 8.65) moves sideways by at most
-// (z0 + r) tan(8.66 div) before it has passed the sample.  With a 1 % and 1 um margin.
+// (z0 + r) tan(8.66 div) before it has passed the sample.  With a 1 % and 1 um margin, and
+// 2^-24 of the beam's width for the rounding of an FP32 position.
 void set_miss_bounds(const mcv::SampleP<double>& S, mcv::BeamP<double>* B) {
-  B->x_safe = INFINITY;
-  B->y_safe = INFINITY;
+  no_miss_bounds(B);
   // only for a start plane upstream of the sample centre and energies that are all positive
   if (!B->energy_positive || !(B->z0 >= 0.0)) return;
   double r = 0.0, hh = 0.0;
@@ -315,8 +321,15 @@ void set_miss_bounds(const mcv::SampleP<double>& S, mcv::BeamP<double>* B) {
   const double a = 8.66 * B->div;
   if (!(a < 1.0)) return;
   const double shift = (B->z0 + r) * std::tan(a) * 1.01 + 1e-6;
-  B->x_safe = r + shift;
-  B->y_safe = hh + shift;
+  // |u - 1/2| width > r + shift, as bounds of the uniform's leading 32 bits
+  auto bound = [](double safe, double width, uint32_t* lo, uint32_t* hi) {
+    if (!(safe < 0.5 * width)) return;
+    const double f = safe / width, scale = 4294967296.0;
+    *lo = (uint32_t)std::max(0.0, std::floor((0.5 - f) * scale) - 260.0);
+    *hi = (uint32_t)std::min(scale - 1.0, std::ceil((0.5 + f) * scale) + 260.0);
+  };
+  bound(r + shift, B->width, &B->fx_lo, &B->fx_hi);
+  bound(hh + shift, B->height, &B->fy_lo, &B->fy_hi);
 }
 
 // radius of a cylinder about the y axis that holds every scatterer of the sample
@@ -384,11 +397,10 @@ void cast_beam(const mcv::BeamP<double>& d, mcv::BeamP<float>* f) {
   f->t0_hi = d.t0_hi;
   f->t0_lo = d.t0_lo;
   f->energy_positive = d.energy_positive;
-  // rounded up: the float bounds stay on the safe side
-  f->x_safe = (float)d.x_safe;
-  if ((double)f->x_safe < d.x_safe) f->x_safe = std::nextafter(f->x_safe, INFINITY);
-  f->y_safe = (float)d.y_safe;
-  if ((double)f->y_safe < d.y_safe) f->y_safe = std::nextafter(f->y_safe, INFINITY);
+  f->fx_lo = d.fx_lo;
+  f->fx_hi = d.fx_hi;
+  f->fy_lo = d.fy_lo;
+  f->fy_hi = d.fy_hi;
 }
 
 void cast_sample(const mcv::SampleP<double>& d, mcv::SampleP<float>* f) {

@@ -15,7 +15,8 @@ using namespace mcv::host;
 
 namespace {
 
-constexpr int kWarpsPerBlock = 4;  // the kernels' 128 threads
+// warps of a block of the batched kernel (WaveCfg)
+int warps_per_block(int fp_mode) { return mcv::wave_threads(fp_mode) / 32; }
 constexpr int64_t kDefaultChunk = 8192;
 constexpr int64_t kMinChunk = 256;
 
@@ -179,7 +180,8 @@ int64_t default_chunk(int64_t total_n, int64_t warps) {
   return (c / 32) * 32;
 }
 
-int grid_of(int sm_count, int blocks_per_sm, int64_t n_items) {
+int grid_of(int fp_mode, int sm_count, int blocks_per_sm, int64_t n_items) {
+  const int kWarpsPerBlock = warps_per_block(fp_mode);
   const int64_t full = (int64_t)sm_count * blocks_per_sm;
   const int64_t need = (n_items + kWarpsPerBlock - 1) / kWarpsPerBlock;
   return (int)std::max<int64_t>(1, std::min(full, need));
@@ -216,7 +218,7 @@ mcv_status upload(mcv_batch* b) {
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy (batch parameters)");
   point_args(b->d_block, b->im, b->chunk, &b->Q);
   b->n_items = count_items(b->im.n, b->chunk);
-  b->grid = grid_of(b->ctx->sm_count, b->blocks_per_sm, b->n_items);
+  b->grid = grid_of(b->im.fp, b->ctx->sm_count, b->blocks_per_sm, b->n_items);
   return MCV_OK;
 }
 
@@ -272,7 +274,7 @@ mcv_status mcv_batch_create(mcv_ctx* ctx, const mcv_sim* sims, int nsims,
   } else {
     b->blocks_per_sm = b->max_blocks_per_sm;
     b->chunk = default_chunk(b->im.total_n,
-                             (int64_t)ctx->sm_count * b->blocks_per_sm * kWarpsPerBlock);
+                             (int64_t)ctx->sm_count * b->blocks_per_sm * warps_per_block(b->im.fp));
   }
   cudaError_t e = cudaMalloc(&b->d_block, device_bytes(b->im));
   if (e != cudaSuccess) {
@@ -380,7 +382,7 @@ mcv_status mcv_batch_tune(mcv_batch* b, int64_t trial_neutrons, void* stream) {
     point_args(d_trial, tr, tc, &Q);
     const int64_t items = count_items(tr.n, tc);
     for (int bps = b->max_blocks_per_sm; bps >= std::max(1, b->max_blocks_per_sm - 1); --bps) {
-      const int grid = grid_of(b->ctx->sm_count, bps, items);
+      const int grid = grid_of(b->im.fp, b->ctx->sm_count, bps, items);
       st = launch(b, Q, items, grid, s);  // warm-up
       if (st != MCV_OK) break;
       e = cudaEventRecord(ev0, s);
@@ -434,7 +436,7 @@ mcv_status mcv_trace_batch(mcv_ctx* ctx, const mcv_sim* sims, int nsims,
     b.blocks_per_sm = std::min(t.blocks_per_sm, b.max_blocks_per_sm);
   } else {
     b.blocks_per_sm = b.max_blocks_per_sm;
-    b.chunk = default_chunk(b.im.total_n, (int64_t)ctx->sm_count * b.blocks_per_sm * kWarpsPerBlock);
+    b.chunk = default_chunk(b.im.total_n, (int64_t)ctx->sm_count * b.blocks_per_sm * warps_per_block(b.im.fp));
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const std::vector<unsigned char> img = device_image(b.im);
@@ -446,7 +448,7 @@ mcv_status mcv_trace_batch(mcv_ctx* ctx, const mcv_sim* sims, int nsims,
   if (e == cudaSuccess) {
     point_args(d, b.im, b.chunk, &b.Q);
     const int64_t items = count_items(b.im.n, b.chunk);
-    st = launch(&b, b.Q, items, grid_of(ctx->sm_count, b.blocks_per_sm, items), s);
+    st = launch(&b, b.Q, items, grid_of(b.im.fp, ctx->sm_count, b.blocks_per_sm, items), s);
   }
   cudaError_t ef = cudaFreeAsync(d, s);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync (batch parameters)");

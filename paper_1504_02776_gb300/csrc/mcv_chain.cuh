@@ -5,8 +5,6 @@
 //
 // Policy interface (device, per lane):
 //   kWantsGs                        compile-time: path lengths in scatterer A.gs are needed
-//   kMeetingOnly                    compile-time: only neutrons that meet the sample matter
-//                                   (their other packets carry nothing the policy uses)
 //   start(L)                        a new neutron begins
 //   emit(A, tu, rng, L, we, atten, lg)   packet of order L.o with weight we = w e^{-tau}
 //   scatter(A, L, j, a_fac, out, lg_pt, speed_in)  after the kernel of order L.o scattered
@@ -32,7 +30,7 @@ __device__ __forceinline__ bool load_input(const TraceArgs& A, int64_t i, Ray<R>
   const R vy = static_cast<const R*>(A.in_vy)[i];
   const R vz = static_cast<const R*>(A.in_vz)[i];
   const R sp = Mth<R>::sqrt(vx * vx + vy * vy + vz * vz);
-  if (!(sp > R(0))) return false;
+  if (!Mth<R>::positive(sp)) return false;
   n->x = static_cast<const R*>(A.in_x)[i];
   n->y = static_cast<const R*>(A.in_y)[i];
   n->z = static_cast<const R*>(A.in_z)[i];
@@ -131,7 +129,7 @@ __device__ __forceinline__ bool step_scatter(const TraceArgs& A, const SampleP<R
     if (k < st.ns && !found) {
       const R len = st.seg[k].b - st.seg[k].a;
       const R m = pick_mu<R, NS>(st.mu, st.seg[k].j);
-      if (ell < acc + len || k == st.ns - 1) {
+      if (M::lt_nonneg(ell, acc + len) || k == st.ns - 1) {
         const R part = ell - acc;
         s_pt = st.seg[k].a + part;
         tau_pt += m * part;
@@ -152,7 +150,7 @@ __device__ __forceinline__ bool step_scatter(const TraceArgs& A, const SampleP<R
   L.n.y += s_pt * L.n.dy;
   L.n.z += s_pt * L.n.dz;
   L.n.t.add(M::div(s_pt, L.n.speed));
-  const int kk = (sc.nk == 2 && !(u_k * sc.ksig_sum < sc.ksig0)) ? 1 : 0;
+  const int kk = (sc.nk == 2 && !M::lt_nonneg(u_k * sc.ksig_sum, sc.ksig0)) ? 1 : 0;
   Scatter<R> out;
   const bool ok = scatter_kernel<R, KS>(S, sc, kk, rng, L.o, &L.n, &out, &pol.err);
   if (!ok) {
@@ -162,26 +160,11 @@ __device__ __forceinline__ bool step_scatter(const TraceArgs& A, const SampleP<R
   L.n.w = L.n.w * a_fac * out.factor;
   pol.scatter(A, L, j, a_fac, out, lg_pt, speed_in);
   L.o += 1;
-  if (L.n.w < S.min_prob || (A.stop_on_zero && L.n.w == R(0))) {
+  if (M::lt(L.n.w, S.min_prob) || (A.stop_on_zero && M::is_zero(L.n.w))) {
     pol.clear(A, L.idx, L.o);
     return false;
   }
   return true;
-}
-
-// The source draw of a neutron that matters only if it meets the sample: false as soon as
-// the footprint (host-derived sure-miss bounds) or the direction shows that it misses, which
-// skips the later draws; otherwise the same packet as make_beam.
-template <typename R, int NS, class Rng>
-__device__ __forceinline__ bool make_beam_meeting(const BeamP<R>& B, const SampleP<R>& S,
-                                                  const Rng& rng, Ray<R>* n) {
-  R aux;
-  beam_footprint(B, rng, n);
-  if (surely_misses<R>(B, *n)) return false;
-  beam_divergence(B, rng, n, &aux);
-  Seg<R> seg[2 * NS];
-  if (assembly_segs<R, NS>(S, *n, seg) == 0) return false;
-  return beam_energy(B, rng, aux, n);
 }
 
 // One order of one neutron: segments ahead, emission of the transmitted packet, then the
@@ -193,7 +176,7 @@ __device__ __forceinline__ bool chain_step(const TraceArgs& A, const R* tu, Lane
   StepState<R, NS> st;
   const R we = step_segments<R, NS, P::kWantsGs>(A, S, L, st);
   pol.emit(A, tu, rng, L, we, st.atten, st.lg, st.len_tot);
-  if (L.o == S.max_orders || !(st.len_tot > R(0))) {
+  if (L.o == S.max_orders || !Mth<R>::positive(st.len_tot)) {
     pol.clear(A, L.idx, L.o + 1);
     return false;
   }
@@ -202,8 +185,7 @@ __device__ __forceinline__ bool chain_step(const TraceArgs& A, const R* tu, Lane
 
 // Warp loop: each warp owns ids [lo, hi) of the launch; lanes whose neutron finished take
 // the next ids at the top of each step, again while some lane is still without a live
-// neutron (a policy that keeps only the neutrons meeting the sample drops two thirds of its
-// draws), so all 32 lanes run chain_step together.
+// neutron, so all 32 lanes run chain_step together.
 template <typename R, int NS, int DET, int KS, class P>
 __device__ __forceinline__ void run_chain(const TraceArgs& A, const R* tu, P& pol) {
   const unsigned kFull = 0xffffffffu;
@@ -233,8 +215,7 @@ __device__ __forceinline__ void run_chain(const TraceArgs& A, const R* tu, P& po
             ok = load_input<R>(A, i, &L.n);
           } else {
             const NeutronRng rng(A.keys, L.nid);
-            ok = P::kMeetingOnly ? make_beam_meeting<R, NS>(Bof<R>(A), Sof<R>(A), rng, &L.n)
-                                 : make_beam<R>(Bof<R>(A), rng, &L.n);
+            ok = make_beam<R>(Bof<R>(A), rng, &L.n);
           }
           ok = ok && !(L.n.w < Sof<R>(A).min_prob) && !(A.stop_on_zero && L.n.w == R(0));
           if (!ok) pol.clear(A, i, 0);

@@ -22,6 +22,25 @@ struct Mth;
 template <>
 struct Mth<float> {
   static __device__ __forceinline__ float div(float a, float b) { return a / b; }
+  static __device__ __forceinline__ float norm2(float x, float z) { return __fmaf_rn(z, z, __fmul_rn(x, x)); }
+  // a divisor of several quotients (FP64: its reciprocal)
+  using Rcp = float;
+  static __device__ __forceinline__ float rcp(float b) { return b; }
+  static __device__ __forceinline__ float divr(float a, float r) { return a / r; }
+  static __device__ __forceinline__ bool lt(float a, float b) { return a < b; }
+  static __device__ __forceinline__ bool le(float a, float b) { return a <= b; }
+  static __device__ __forceinline__ bool lt_nonneg(float a, float b) { return a < b; }
+  static __device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+  static __device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
+  // floor(x) where 0 <= x < n, else -1
+  static __device__ __forceinline__ int index_below(float x, int n) {
+    const float f = floorf(x);
+    return (f >= 0.0f && f < (float)n) ? (int)f : -1;
+  }
+  // floor(x) clamped to 0 .. n - 1
+  static __device__ __forceinline__ int index_clamped(float x, int n) {
+    return min(max((int)floorf(x), 0), n - 1);
+  }
   static __device__ __forceinline__ float sqrt(float x) { return sqrtf(x); }
   // exp and log from the hardware approximations (a few ulp; subnormals kept, so a tiny
   // table value or weight is not flushed to zero)
@@ -57,6 +76,25 @@ struct Mth<double> {
   // on the integer pipes (mcv_soft64.cuh): division and square root with the FP64 pipe's
   // results, the elementary functions at least as accurate as the library's
   static __device__ __forceinline__ double div(double a, double b) { return soft64::div(a, b); }
+  static __device__ __forceinline__ double norm2(double x, double z) { return x * x + z * z; }
+  using Rcp = soft64::Recip;
+  static __device__ __forceinline__ Rcp rcp(double b) { return Rcp{b, soft64::recip_of(b)}; }
+  static __device__ __forceinline__ double divr(double a, const Rcp& r) {
+    return soft64::div_by(a, r.b, r.y);
+  }
+  static __device__ __forceinline__ bool lt(double a, double b) { return a < b; }
+  static __device__ __forceinline__ bool le(double a, double b) { return a <= b; }
+  static __device__ __forceinline__ bool lt_nonneg(double a, double b) {
+    return soft64::lt_nonneg(a, b);
+  }
+  static __device__ __forceinline__ bool positive(double x) { return soft64::positive(x); }
+  static __device__ __forceinline__ bool is_zero(double x) { return soft64::is_zero(x); }
+  static __device__ __forceinline__ int index_below(double x, int n) {
+    return soft64::index_below(x, n);
+  }
+  static __device__ __forceinline__ int index_clamped(double x, int n) {
+    return soft64::index_clamped(x, n);
+  }
   static __device__ __forceinline__ double sqrt(double x) { return soft64::sqrt(x); }
   static __device__ __forceinline__ double exp(double x) { return soft64::exp(x); }
   static __device__ __forceinline__ double log(double x) { return soft64::log(x); }
@@ -125,21 +163,18 @@ __device__ __forceinline__ R to_unit(uint32_t hi, uint32_t lo);
 
 template <>
 __device__ __forceinline__ double to_unit<double>(uint32_t hi, uint32_t lo) {
-  const uint64_t k = ((uint64_t)hi << 21) | (uint64_t)(lo >> 11);
-  return __fma_rn((double)k, 0x1p-53, 0x1p-54);
+  return soft64::uniform53(hi, lo);
 }
 
-// FP32: the same 53-bit number rounded to float, built on the integer and FP32 pipes only
-// (exact small-integer to float through the 2^23 bias; one rounding in the final FMA).
-__device__ __forceinline__ float small_int_to_float(uint32_t v) {  // v < 2^23, exact
-  return __int_as_float(0x4b000000u | v) - 8388608.0f;
-}
+// FP32: the same 53-bit number rounded to float
+//   u = (hi 2^21 + (lo >> 11) + 1/2) 2^-53 = hi 2^-32 + c,  c = (2 (lo >> 11) + 1) 2^-54:
+// hi rounded to float, c exact (its 22 bits as a float in [2^23, 2^24), scaled and shifted
+// back by one FMA), one rounding in the final FMA.  Six instructions; hi through its 16-bit
+// halves, and c with separate subtraction and scaling, took thirteen.
 template <>
 __device__ __forceinline__ float to_unit<float>(uint32_t hi, uint32_t lo) {
-  // u = (hi 2^21 + (lo >> 11) + 1/2) 2^-53 = hi 2^-32 + c,  c = (2 (lo >> 11) + 1) 2^-54
-  const float h = __fmaf_rn(small_int_to_float(hi >> 16), 65536.0f, small_int_to_float(hi & 0xffffu));
-  const float c = small_int_to_float(((lo >> 11) << 1) | 1u) * 0x1p-54f;
-  return fminf(__fmaf_rn(h, 0x1p-32f, c), 0x1.fffffep-1f);
+  const float c = __fmaf_rn(__uint_as_float(0x4b000001u | (lo >> 10)), 0x1p-54f, -0x1p-31f);
+  return fminf(__fmaf_rn(__uint2float_rn(hi), 0x1p-32f, c), 0x1.fffffep-1f);
 }
 
 // The stream of one neutron: key (seed, sim) given by its round keys, counter
@@ -151,9 +186,12 @@ struct NeutronRngT {
   __device__ __forceinline__ NeutronRngT(KS keys, int64_t nid)
       : ks(keys), n0((uint32_t)((uint64_t)nid & 0xffffffffu)),
         n1((uint32_t)((uint64_t)nid >> 32)) {}
+  __device__ __forceinline__ Words words(int event, int block) const {
+    return philox10(n0, n1, (uint32_t)(4 * (event + 1) + block), 0u, ks);
+  }
   template <typename R>
   __device__ __forceinline__ void pair(int event, int block, R* u0, R* u1) const {
-    const Words w = philox10(n0, n1, (uint32_t)(4 * (event + 1) + block), 0u, ks);
+    const Words w = words(event, block);
     *u0 = to_unit<R>(w.a, w.b);
     *u1 = to_unit<R>(w.c, w.d);
   }
@@ -237,17 +275,21 @@ __device__ __forceinline__ const BeamP<double>& Bof<double>(const TraceArgs& A) 
 // alone decide whether the neutron meets the sample, and a neutron that misses it needs no
 // energy when every energy draw is positive (BeamP::energy_positive).
 // aux: what the energy part needs from the direction part (FP32: tan^2 ax + tan^2 ay).
-// The footprint alone already settles most misses: a neutron whose footprint lies outside
-// (x_safe, y_safe) cannot reach the sample whatever its divergence (BeamP::x_safe).
-template <class Rng>
-__device__ __forceinline__ void beam_footprint(const BeamP<double>& B,
-                                                       const Rng& rng, Ray<double>* n) {
-  double u0, u1;
-  rng.template pair<double>(-1, 1, &u0, &u1);
-  n->x = (u0 - 0.5) * B.width;
-  n->y = (u1 - 0.5) * B.height;
+// The footprint alone already settles most misses: a neutron whose footprint lies far enough
+// out cannot reach the sample whatever its divergence (footprint_misses).
+template <typename R>
+__device__ __forceinline__ void beam_footprint(const BeamP<R>& B, const Words& w, Ray<R>* n) {
+  n->x = (to_unit<R>(w.a, w.b) - R(0.5)) * B.width;
+  n->y = (to_unit<R>(w.c, w.d) - R(0.5)) * B.height;
   n->z = -B.z0;
-  n->w = 1.0;
+  n->w = R(1);
+}
+
+// Integer tests on the random words: two thirds of a 5 x 5 cm beam end here, before a
+// uniform is formed (FP64: before any FP64 instruction).
+template <typename R>
+__device__ __forceinline__ bool footprint_misses(const BeamP<R>& B, const Words& w) {
+  return w.a < B.fx_lo || w.a > B.fx_hi || w.c < B.fy_lo || w.c > B.fy_hi;
 }
 
 template <class Rng>
@@ -262,9 +304,10 @@ __device__ __forceinline__ void beam_divergence(const BeamP<double>& B,
   const double ax = B.div * (rr * c), ay = B.div * (rr * s);
   const double tx = M::tan(ax), ty = M::tan(ay);
   const double norm = M::sqrt(tx * tx + ty * ty + 1.0);
-  n->dx = M::div(tx, norm);
-  n->dy = M::div(ty, norm);
-  n->dz = M::div(1.0, norm);
+  const M::Rcp rn = M::rcp(norm);
+  n->dx = M::divr(tx, rn);
+  n->dy = M::divr(ty, rn);
+  n->dz = M::divr(1.0, rn);
   *aux = 0.0;
 }
 
@@ -278,7 +321,7 @@ __device__ __forceinline__ bool beam_energy(const BeamP<double>& B,
   M::sincos2pi(u1, &s, &c);
   const double zE = M::sqrt(-2.0 * M::log(u0)) * c;
   const double E = B.ei * (1.0 + B.rel * zE);
-  if (!(E > 0.0)) return false;
+  if (!M::positive(E)) return false;
   n->speed = M::sqrt(M::div(E, kMeVPerV2));
   n->t.set(M::div(B.l1 - B.z0, n->speed * n->dz));
   return true;
@@ -288,17 +331,6 @@ __device__ __forceinline__ bool beam_energy(const BeamP<double>& B,
 // (computed once in FP64 on the host) times small FP32 corrections, so that the FP64 time
 // keeps ~1e-12 s accuracy: speed = v0 (1 + eta), eta = d/(1 + sqrt(1 + d)), d = rel z;
 // path/speed = t0 (1 + xi)/(1 + eta), xi = e/(1 + sqrt(1 + e)), e = tan^2 ax + tan^2 ay.
-template <class Rng>
-__device__ __forceinline__ void beam_footprint(const BeamP<float>& B,
-                                                      const Rng& rng, Ray<float>* n) {
-  float u0, u1;
-  rng.template pair<float>(-1, 1, &u0, &u1);
-  n->x = (u0 - 0.5f) * B.width;
-  n->y = (u1 - 0.5f) * B.height;
-  n->z = -B.z0;
-  n->w = 1.0f;
-}
-
 template <class Rng>
 __device__ __forceinline__ void beam_divergence(const BeamP<float>& B,
                                                        const Rng& rng, Ray<float>* n,
@@ -342,25 +374,19 @@ __device__ __forceinline__ bool beam_energy(const BeamP<float>& B,
 template <typename R, class Rng>
 __device__ __forceinline__ bool make_beam(const BeamP<R>& B, const Rng& rng, Ray<R>* n) {
   R aux;
-  beam_footprint(B, rng, n);
+  beam_footprint(B, rng.words(-1, 1), n);
   beam_divergence(B, rng, n, &aux);
   return beam_energy(B, rng, aux, n);
-}
-
-// the footprint is far enough from the sample that the neutron misses it for any divergence
-template <typename R>
-__device__ __forceinline__ bool surely_misses(const BeamP<R>& B, const Ray<R>& n) {
-  return Mth<R>::fabs(n.x) > B.x_safe || Mth<R>::fabs(n.y) > B.y_safe;
 }
 
 // ---- geometry ----------------------------------------------------------------------------
 // Line r + s d inside the infinite cylinder x^2 + z^2 < rad^2 (axis y): closest-approach
 // form, squared axis distance (r x d)^2 / a with a = dx^2 + dz^2.
-template <typename R>
+template <typename R, bool NORM = false>
 __device__ __forceinline__ bool cyl_span(R rad, R x, R z, R dx, R dz, R* s1, R* s2) {
   using M = Mth<R>;
-  const R a = dx * dx + dz * dz;
-  if (a == R(0)) {
+  const R a = NORM ? M::norm2(dx, dz) : dx * dx + dz * dz;
+  if (M::is_zero(a)) {
     if (x * x + z * z < rad * rad) {
       *s1 = -M::inf();
       *s2 = M::inf();
@@ -368,11 +394,12 @@ __device__ __forceinline__ bool cyl_span(R rad, R x, R z, R dx, R dz, R* s1, R* 
     }
     return false;
   }
-  const R tc = M::div(-(x * dx + z * dz), a);
+  const typename M::Rcp ra = M::rcp(a);
+  const R tc = M::divr(-(x * dx + z * dz), ra);
   const R cr = x * dz - z * dx;
-  const R g = rad * rad - M::div(cr * cr, a);
-  if (!(g > R(0))) return false;
-  const R half = M::sqrt(M::div(g, a));
+  const R g = rad * rad - M::divr(cr * cr, ra);
+  if (!M::positive(g)) return false;
+  const R half = M::sqrt(M::divr(g, ra));
   *s1 = tc - half;
   *s2 = tc + half;
   return true;
@@ -382,7 +409,7 @@ __device__ __forceinline__ bool cyl_span(R rad, R x, R z, R dx, R dz, R* s1, R* 
 template <typename R>
 __device__ __forceinline__ bool slab_span(R half, R p, R dp, R* s1, R* s2) {
   using M = Mth<R>;
-  if (dp == R(0)) {
+  if (M::is_zero(dp)) {
     if (M::fabs(p) < half) {
       *s1 = -M::inf();
       *s2 = M::inf();
@@ -390,7 +417,8 @@ __device__ __forceinline__ bool slab_span(R half, R p, R dp, R* s1, R* s2) {
     }
     return false;
   }
-  const R a = M::div(-half - p, dp), b = M::div(half - p, dp);
+  const typename M::Rcp rp = M::rcp(dp);
+  const R a = M::divr(-half - p, rp), b = M::divr(half - p, rp);
   *s1 = M::fmin(a, b);
   *s2 = M::fmax(a, b);
   return true;
@@ -407,7 +435,7 @@ struct Seg {
 template <typename R>
 __device__ __forceinline__ void put_seg(R a, R b, int j, R s0, Seg<R>* out, int* cnt) {
   const R lo = Mth<R>::fmax(a, s0);
-  if (b > lo) {
+  if (Mth<R>::lt(lo, b)) {
     out[*cnt].a = lo;
     out[*cnt].b = b;
     out[*cnt].j = j;
@@ -431,7 +459,7 @@ __device__ __forceinline__ int shape_segs(const ScatP<R>& S, int j, const Ray<R>
     if (cyl_span<R>((R)S.dim1, n.x, n.z, n.dx, n.dz, &c1, &c2) &&
         slab_span<R>((R)S.half_h, n.y, n.dy, &y1, &y2)) {
       const R lo = M::fmax(c1, y1), hi = M::fmin(c2, y2);
-      if (hi > lo) {
+      if (M::lt(lo, hi)) {
         R i1, i2;
         if (!cyl_span<R>((R)S.dim0, n.x, n.z, n.dx, n.dz, &i1, &i2)) {
           put_seg<R>(lo, hi, j, s0, out, &cnt);
@@ -460,6 +488,117 @@ __device__ __forceinline__ int shape_segs(const ScatP<R>& S, int j, const Ray<R>
   return cnt;
 }
 
+// FP64: the same segments from one function per kind of shape, compiled once per kernel, with
+// the quotients of concentric cylinders and of a slab's two faces sharing their divisor's
+// reciprocal.  Empty segments have a = +inf.
+struct Segs64 {
+  double a0, b0, a1, b1;
+};
+
+static __device__ __forceinline__ void put_seg64(double a, double b, double s0, bool ok,
+                                                 double* oa, double* ob) {
+  const double lo = ::fmax(a, s0);
+  ok = ok && lo < b;
+  *oa = ok ? lo : CUDART_INF;
+  *ob = ok ? b : 0.0;
+}
+
+// cylinder of radius r_out without the one of radius r_in (r_in < 0: solid)
+static __device__ __noinline__ Segs64 cyl_segs64(double r_in, double r_out, double half_h,
+                                                 double x, double y, double z, double dx,
+                                                 double dy, double dz, double s0) {
+  using M = Mth<double>;
+  Segs64 o;
+  o.a0 = o.a1 = CUDART_INF;
+  o.b0 = o.b1 = 0.0;
+  double y1, y2, c1, c2, i1 = 0.0, i2 = 0.0;
+  bool inner = false;
+  if (M::is_zero(dy)) {
+    if (!(::fabs(y) < half_h)) return o;
+    y1 = -CUDART_INF;
+    y2 = CUDART_INF;
+  } else {
+    const M::Rcp ry = M::rcp(dy);
+    const double ya = M::divr(-half_h - y, ry), yb = M::divr(half_h - y, ry);
+    const bool up = !signbit(dy);  // the lower face first
+    y1 = up ? ya : yb;
+    y2 = up ? yb : ya;
+  }
+  const double a = dx * dx + dz * dz;
+  if (M::is_zero(a)) {
+    const double r2 = x * x + z * z;
+    if (!(r2 < r_out * r_out)) return o;
+    c1 = i1 = -CUDART_INF;
+    c2 = i2 = CUDART_INF;
+    inner = r_in >= 0.0 && r2 < r_in * r_in;
+  } else {
+    const M::Rcp ra = M::rcp(a);
+    const double cr = x * dz - z * dx;
+    const double d2 = M::divr(cr * cr, ra);
+    const double g = r_out * r_out - d2, gi = r_in * r_in - d2;
+    if (!M::positive(g)) return o;
+    const double tc = M::divr(-(x * dx + z * dz), ra);
+    const double h = M::sqrt(M::divr(g, ra));
+    c1 = tc - h;
+    c2 = tc + h;
+    inner = M::positive(gi) && M::positive(r_in);
+    if (inner) {
+      const double hi = M::sqrt(M::divr(gi, ra));
+      i1 = tc - hi;
+      i2 = tc + hi;
+    }
+  }
+  const double lo = ::fmax(c1, y1), hi = ::fmin(c2, y2);
+  const bool ok = lo < hi;
+  put_seg64(lo, inner ? ::fmin(hi, i1) : hi, s0, ok, &o.a0, &o.b0);
+  put_seg64(::fmax(lo, i2), hi, s0, ok && inner, &o.a1, &o.b1);
+  return o;
+}
+
+// box of half sides hx, hy, hz in its own frame: one segment (a, b)
+static __device__ __noinline__ double2 box_seg64(double hx, double hy, double hz, double x,
+                                                 double y, double z, double dx, double dy,
+                                                 double dz, double s0) {
+  double a = 0.0, b = 0.0, lo = -CUDART_INF, hi = CUDART_INF;
+  bool ok = slab_span<double>(hx, x, dx, &a, &b);
+  lo = ::fmax(lo, a);
+  hi = ::fmin(hi, b);
+  ok = ok && slab_span<double>(hy, y, dy, &a, &b);
+  lo = ::fmax(lo, a);
+  hi = ::fmin(hi, b);
+  ok = ok && slab_span<double>(hz, z, dz, &a, &b);
+  lo = ::fmax(lo, a);
+  hi = ::fmin(hi, b);
+  put_seg64(lo, hi, s0, ok, &a, &b);
+  return make_double2(a, b);
+}
+
+__device__ __forceinline__ int shape_segs64(const ScatP<double>& S, int j, const Ray<double>& n,
+                                            Seg<double>* out, double s0) {
+  out[0].j = out[1].j = j;
+  out[1].a = CUDART_INF;
+  out[1].b = 0.0;
+  if (S.shape == MCV_SHAPE_BLOCK) {
+    const double c = S.cos_rot, s = S.sin_rot;
+    const double2 g = box_seg64(0.5 * S.dim0, 0.5 * S.dim1, 0.5 * S.dim2, c * n.x - s * n.z, n.y,
+                                s * n.x + c * n.z, c * n.dx - s * n.dz, n.dy,
+                                s * n.dx + c * n.dz, s0);
+    out[0].a = g.x;
+    out[0].b = g.y;
+    return soft64::lt_nonneg(g.x, CUDART_INF) ? 1 : 0;
+  }
+  const bool hollow = S.shape == MCV_SHAPE_HOLLOW_CYL;
+  const Segs64 g = cyl_segs64(hollow ? S.dim0 : -1.0, hollow ? S.dim1 : S.dim0, S.half_h, n.x, n.y,
+                              n.z, n.dx, n.dy, n.dz, s0);
+  const bool has0 = soft64::lt_nonneg(g.a0, CUDART_INF), has1 = soft64::lt_nonneg(g.a1, CUDART_INF);
+  // the segments packed to the front, as put_seg leaves them
+  out[0].a = has0 ? g.a0 : g.a1;
+  out[0].b = has0 ? g.b0 : g.b1;
+  out[1].a = has0 ? g.a1 : CUDART_INF;
+  out[1].b = has0 ? g.b1 : 0.0;
+  return (has0 ? 1 : 0) + (has1 ? 1 : 0);
+}
+
 // All segments ahead in the sample assembly, sorted by entry (ray tracing in a composite,
 // section 2.4.3).  NS = number of scatterers (compile time); unused entries get a = +inf.
 template <typename R, int NS>
@@ -474,7 +613,13 @@ __device__ __forceinline__ int assembly_segs(const SampleP<R>& S, const Ray<R>& 
     two[1].a = M::inf();
     two[0].b = two[1].b = R(0);
     two[0].j = two[1].j = j;
-    const int c = (j < S.ns) ? shape_segs<R>(S.s[j], j, n, two, s0) : 0;
+    int c = 0;
+    if (j < S.ns) {
+      if constexpr (sizeof(R) == 8)
+        c = shape_segs64(S.s[j], j, n, two, s0);
+      else
+        c = shape_segs<R>(S.s[j], j, n, two, s0);
+    }
     seg[2 * j] = two[0];
     seg[2 * j + 1] = two[1];
     total += c;
@@ -484,7 +629,7 @@ __device__ __forceinline__ int assembly_segs(const SampleP<R>& S, const Ray<R>& 
   for (int pass = 0; pass < 2 * NS; ++pass) {
 #pragma unroll
     for (int i = (pass & 1); i + 1 < 2 * NS; i += 2) {
-      if (seg[i].a > seg[i + 1].a) {
+      if (M::lt(seg[i + 1].a, seg[i].a)) {
         const Seg<R> t = seg[i];
         seg[i] = seg[i + 1];
         seg[i + 1] = t;
@@ -519,7 +664,7 @@ __device__ __forceinline__ void turn(R c, R s, R u, R* dx, R* dy, R* dz) {
   using M = Mth<R>;
   const R x = *dx, y = *dy, z = *dz;
   R e1x, e1y, e1z;
-  if (M::fabs(z) < R(0.9)) {  // (0,0,1) x d
+  if (M::lt_nonneg(M::fabs(z), R(0.9))) {  // (0,0,1) x d
     e1x = -y;
     e1y = x;
     e1z = R(0);
@@ -570,33 +715,34 @@ __device__ __forceinline__ bool kernel_sqe(const SampleP<R>& S, const Rng& rng, 
   const R Ei = (R)kMeVPerV2 * n->speed * n->speed;
   const R ki = (R)kKPerV * n->speed;
   const R e_lo = (R)S.e_min, e_hi = M::fmin((R)S.e_max, Ei);
-  if (!(e_hi > e_lo)) return false;
+  if (!M::lt(e_lo, e_hi)) return false;
   const R dE = e_hi - e_lo;
   R u0, u1;
   rng.template pair<R>(o, 1, &u0, &u1);
   const R E = e_lo + u0 * dE;
   // Ef = Ei - E; when the range ends at Ei it is the sampled offset from that end
-  const R Ef = (e_hi == Ei) ? (R(1) - u0) * dE : Ei - E;
-  if (!(Ef > R(0))) return false;
+  const R Ef = M::le(Ei, e_hi) ? (R(1) - u0) * dE : Ei - E;
+  if (!M::positive(Ef)) return false;
   const R speed_f = M::sqrt(M::div(Ef, (R)kMeVPerV2));
   const R kf = (R)kKPerV * speed_f;
   const R q_lo = M::fabs(ki - kf);
   const R q_hi = M::fmin(ki + kf, (R)S.q_max);
-  if (!(q_hi > q_lo)) return false;
+  if (!M::lt(q_lo, q_hi)) return false;
   const R dQ = q_hi - q_lo;
   const R Q = q_lo + u1 * dQ;
   // cos and sin of the scattering angle from 1 -/+ cos, each a product whose small factor
   // is the sampled offset from an end of the Q range (no cancellation near 0 or pi)
-  const R den = R(2) * ki * kf;
-  const R one_m = M::div((u1 * dQ) * (Q + q_lo), den);
-  const R top = (q_hi == ki + kf) ? (R(1) - u1) * dQ : (ki + kf) - Q;
-  const R one_p = M::div(top * (ki + kf + Q), den);
-  R c2t = (one_m <= one_p) ? R(1) - one_m : one_p - R(1);
+  const typename M::Rcp den = M::rcp(R(2) * ki * kf);
+  const R one_m = M::divr((u1 * dQ) * (Q + q_lo), den);
+  const R top = M::le(ki + kf, q_hi) ? (R(1) - u1) * dQ : (ki + kf) - Q;
+  const R one_p = M::divr(top * (ki + kf + Q), den);
+  R c2t = M::le(one_m, one_p) ? R(1) - one_m : one_p - R(1);
   c2t = M::fmin(R(1), M::fmax(R(-1), c2t));
   const R s2t = M::sqrt(M::fmax(R(0), one_m * one_p));
-  const R fq = M::floor(M::div(Q, (R)S.dq)), fe = M::floor(M::div(E - (R)S.e_min, (R)S.de));
-  if (!(fq >= R(0) && fq < (R)S.nq && fe >= R(0) && fe < (R)S.ne)) return false;
-  const int entry = (int)fq * S.ne + (int)fe;
+  const int iq = M::index_below(M::div(Q, (R)S.dq), S.nq);
+  const int ie = M::index_below(M::div(E - (R)S.e_min, (R)S.de), S.ne);
+  if (iq < 0 || ie < 0) return false;
+  const int entry = iq * S.ne + ie;
   if (entry < 0 || entry >= S.nq * S.ne) {
     *err = 1;
     return false;
@@ -631,7 +777,7 @@ __device__ __forceinline__ int draw_mass(const R* __restrict__ cdf, int size, R 
   int lo = 0, hi = size;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (__ldg(cdf + mid) > x) hi = mid;
+    if (Mth<R>::lt_nonneg(x, __ldg(cdf + mid))) hi = mid;
     else lo = mid + 1;
   }
   return lo < size - 1 ? lo : size - 1;
@@ -648,7 +794,7 @@ __device__ __forceinline__ bool kernel_phonon(const SampleP<R>& S, const Rng& rn
   rng.template pair<R>(o, 2, &u2, &u3);
   sc->entry = -1;
   sc->s_value = R(1);
-  if (u0 < S.ph_p0) {
+  if (M::lt_nonneg(u0, S.ph_p0)) {
     // elastic: isotropic direction, speed unchanged
     const R ct = R(2) * u2 - R(1);
     const R st = R(2) * M::sqrt(u2 * (R(1) - u2));
@@ -666,7 +812,7 @@ __device__ __forceinline__ bool kernel_phonon(const SampleP<R>& S, const Rng& rn
     sc->e = R(0);
     return true;
   }
-  const bool one = u0 < S.ph_p01;
+  const bool one = M::lt_nonneg(u0, S.ph_p01);
   const R p_ch = one ? S.ph_p1 : S.ph_p2;
   const R ue = M::div(u0 - (one ? S.ph_p0 : S.ph_p01), p_ch);
   // one search for both channels (the lanes of a warp pick either), from A_1 or from B
@@ -675,17 +821,17 @@ __device__ __forceinline__ bool kernel_phonon(const SampleP<R>& S, const Rng& rn
   const R mass = one ? R(1) : __ldg(S.ph_b + k);
   const R E = ((R)i + (u1 - R(0.5))) * S.ph_de;
   const R Ef = Ei - E;
-  if (!(Ef > R(0))) return false;
+  if (!M::positive(Ef)) return false;
   const R speed_f = M::sqrt(M::div(Ef, (R)kMeVPerV2));
   const R kf = (R)kKPerV * speed_f;
   const R q_lo = M::fabs(ki - kf), q_hi = ki + kf;
   const R dQ = q_hi - q_lo;
   const R Q = q_lo + u2 * dQ;
   // scattering angle from 1 -/+ cos as products of the offsets from the ends of the range
-  const R den = R(2) * ki * kf;
-  const R one_m = M::div((u2 * dQ) * (Q + q_lo), den);
-  const R one_p = M::div(((R(1) - u2) * dQ) * (ki + kf + Q), den);
-  R c2t = (one_m <= one_p) ? R(1) - one_m : one_p - R(1);
+  const typename M::Rcp den = M::rcp(R(2) * ki * kf);
+  const R one_m = M::divr((u2 * dQ) * (Q + q_lo), den);
+  const R one_p = M::divr(((R(1) - u2) * dQ) * (ki + kf + Q), den);
+  R c2t = M::le(one_m, one_p) ? R(1) - one_m : one_p - R(1);
   c2t = M::fmin(R(1), M::fmax(R(-1), c2t));
   const R s2t = M::sqrt(M::fmax(R(0), one_m * one_p));
   // the term of S at (Q, E) over the sampling mass of E
@@ -727,17 +873,18 @@ __device__ __forceinline__ bool kernel_bragg(const SampleP<R>& S, R sig_k, const
   using M = Mth<R>;
   const R ki = (R)kKPerV * n->speed;
   const R lam = M::div(R(2.0 * kPi), ki);
+  const R half_lam = R(0.5) * lam;
   int lo = 0, hi = S.n_refl;  // allowed: the reflections with lam < 2 d
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (lam < R(2) * __ldg(S.refl_d + mid)) lo = mid + 1;
+    if (M::lt_nonneg(half_lam, __ldg(S.refl_d + mid))) lo = mid + 1;
     else hi = mid;
   }
   const int allowed = lo;
   if (allowed == 0) return false;
   const R csum = __ldg(S.refl_c + allowed - 1);
   const R total = R(0.5) * lam * lam * csum;
-  if (!(total > R(0))) return false;
+  if (!M::positive(total)) return false;
   R u0, u1;
   rng.template pair<R>(o, 1, &u0, &u1);
   const R x = u0 * csum;
@@ -745,7 +892,7 @@ __device__ __forceinline__ bool kernel_bragg(const SampleP<R>& S, R sig_k, const
   hi = allowed - 1;  // the first reflection whose prefix sum exceeds x (the last if none)
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (x < __ldg(S.refl_c + mid)) hi = mid;
+    if (M::lt_nonneg(x, __ldg(S.refl_c + mid))) hi = mid;
     else lo = mid + 1;
   }
   const int pick = lo;
@@ -1002,7 +1149,7 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
   for (int k = 0; k <= kM; ++k) {
     const BvkPoint<R> P = bvk_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz,
                                        lo + (R)k * step, b, sg);
-    if (P.g > R(0)) pos |= (uint64_t)1 << k;
+    if (M::positive(P.g)) pos |= (uint64_t)1 << k;
   }
   const uint64_t change = (pos ^ (pos >> 1)) & ((((uint64_t)1) << kM) - 1);
   const int nroots = __popcll(change);
@@ -1019,7 +1166,7 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
     const R mid = R(0.5) * (ea + eb);
     const BvkPoint<R> P = bvk_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz,
                                        mid, b, sg);
-    if ((P.g > R(0)) == ga_pos)
+    if (M::positive(P.g) == ga_pos)
       ea = mid;
     else
       eb = mid;
@@ -1122,7 +1269,7 @@ __device__ __forceinline__ bool kernel_disp(const SampleP<R>& S, R crot, R srot,
   for (int k = 0; k <= kM; ++k) {
     const DispPoint<R> P = disp_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy,
                                          dfz, lo + (R)k * step);
-    if (P.g > R(0)) pos |= (uint64_t)1 << k;
+    if (M::positive(P.g)) pos |= (uint64_t)1 << k;
   }
   const uint64_t change = (pos ^ (pos >> 1)) & ((((uint64_t)1) << kM) - 1);
   const int nroots = __popcll(change);
@@ -1139,7 +1286,7 @@ __device__ __forceinline__ bool kernel_disp(const SampleP<R>& S, R crot, R srot,
     const R mid = R(0.5) * (ea + eb);
     const DispPoint<R> P = disp_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy,
                                          dfz, mid);
-    if ((P.g > R(0)) == ga_pos)
+    if (M::positive(P.g) == ga_pos)
       ea = mid;
     else
       eb = mid;
@@ -1183,30 +1330,43 @@ struct Hit {
 };
 
 // larger root of the ray with the origin-centred cylinder (the ray starts inside it)
-template <typename R>
+template <typename R, bool NORM>
 __device__ __forceinline__ bool exit_cyl(R rad, const Ray<R>& n, R* s) {
   R s1, s2;
-  if (!cyl_span<R>(rad, n.x, n.z, n.dx, n.dz, &s1, &s2)) return false;
-  if (!(s2 > R(0)) || s2 == Mth<R>::inf()) return false;
+  if (!cyl_span<R, NORM>(rad, n.x, n.z, n.dx, n.dz, &s1, &s2)) return false;
+  if (!Mth<R>::positive(s2) || !Mth<R>::lt(s2, Mth<R>::inf())) return false;
   *s = s2;
   return true;
 }
 
 // Chord of a vertical tube (axis through R (ux, uz)) in coordinates along / across the
 // tube direction, so the large distance R cancels once.
-template <typename R>
+template <typename R, bool NORM = false, int FORM = 0>
 __device__ __forceinline__ bool tube_span(R Rad, R ux, R uz, R rt, const Ray<R>& n, R* s1, R* s2) {
-  const R a = n.dx * n.dx + n.dz * n.dz;
-  if (a == R(0)) return false;
+  const R a = NORM ? Mth<R>::norm2(n.dx, n.dz) : n.dx * n.dx + n.dz * n.dz;
+  if (Mth<R>::is_zero(a)) return false;
+  const typename Mth<R>::Rcp ra = Mth<R>::rcp(a);
   const R o_rad = n.x * ux + n.z * uz - Rad;
   const R o_tan = n.x * uz - n.z * ux;
   const R d_rad = n.dx * ux + n.dz * uz;
   const R d_tan = n.dx * uz - n.dz * ux;
-  const R tc = Mth<R>::div(-(o_rad * d_rad + o_tan * d_tan), a);
+  const R tc = Mth<R>::divr(-(o_rad * d_rad + o_tan * d_tan), ra);
   const R cr = o_rad * d_tan - o_tan * d_rad;
-  const R g = rt * rt - Mth<R>::div(cr * cr, a);
-  if (!(g > R(0))) return false;
-  const R half = Mth<R>::sqrt(Mth<R>::div(g, a));
+  R g;
+  if constexpr (sizeof(R) == 4 && FORM != 0) {
+    // a chord next to the tube's edge is its rounding: held in the kernel's form
+    if constexpr (FORM == 1) {
+      g = __fmaf_rn(rt, rt, -(cr * cr / a));
+    } else {
+      float ia;
+      asm("rcp.approx.f32 %0, %1;" : "=f"(ia) : "f"(a));
+      g = __fmaf_rn(-__fmul_rn(cr, cr), ia, __fmul_rn(rt, rt));
+    }
+  } else {
+    g = rt * rt - Mth<R>::divr(cr * cr, ra);
+  }
+  if (!Mth<R>::positive(g)) return false;
+  const R half = Mth<R>::sqrt(Mth<R>::divr(g, ra));
   *s1 = tc - half;
   *s2 = tc + half;
   return true;
@@ -1218,9 +1378,7 @@ template <typename R>
 __device__ __forceinline__ int64_t tof_bin(const TofWin& W, const Tof<R>& tof);
 template <>
 __device__ __forceinline__ int64_t tof_bin<double>(const TofWin& W, const Tof<double>& tof) {
-  const double fb = ::floor(soft64::div(tof.v - W.tof_min, W.dt));
-  if (!(fb >= 0.0 && fb < (double)W.n_tof)) return -1;
-  return (int64_t)fb;
+  return soft64::index_below(soft64::div(tof.v - W.tof_min, W.dt), W.n_tof);
 }
 template <>
 __device__ __forceinline__ int64_t tof_bin<float>(const TofWin& W, const Tof<float>& tof) {
@@ -1230,7 +1388,7 @@ __device__ __forceinline__ int64_t tof_bin<float>(const TofWin& W, const Tof<flo
   return (int64_t)fb;
 }
 
-template <typename R>
+template <typename R, bool NORM>
 __device__ __forceinline__ Hit<R> detect_surface(const DetP<R>& D, const TofWin& W,
                                                  const Ray<R>& n) {
   using M = Mth<R>;
@@ -1241,16 +1399,14 @@ __device__ __forceinline__ Hit<R> detect_surface(const DetP<R>& D, const TofWin&
   h.w_det = R(0);
   h.pabs = R(0);
   R s;
-  if (!exit_cyl<R>((R)D.radius, n, &s)) return h;
+  if (!exit_cyl<R, NORM>((R)D.radius, n, &s)) return h;
   const R yh = n.y + s * n.dy;
   const R half = (R)D.half_h;
-  if (yh < -half || yh >= half) return h;
+  if (M::lt(yh, -half) || M::le(half, yh)) return h;
   const R xh = n.x + s * n.dx, zh = n.z + s * n.dz;
   const R phi = M::atan2(xh, zh);
-  int ip = (int)M::floor(M::div(phi + (R)kPi, (R)(2.0 * kPi)) * (R)D.n_phi);
-  ip = min(max(ip, 0), D.n_phi - 1);
-  int iy = (int)M::floor(M::div(yh + half, (R)D.height) * (R)D.n_y);
-  iy = min(max(iy, 0), D.n_y - 1);
+  const int ip = M::index_clamped(M::div(phi + (R)kPi, (R)(2.0 * kPi)) * (R)D.n_phi, D.n_phi);
+  const int iy = M::index_clamped(M::div(yh + half, (R)D.height) * (R)D.n_y, D.n_y);
   h.pixel = ip * D.n_y + iy;
   h.tof.add(M::div(s, n.speed));
   h.w_det = n.w;
@@ -1286,18 +1442,18 @@ __device__ __forceinline__ bool det_surely_misses(const DetP<R>& D, const Ray<R>
 // Where a packet meets the tube rows: the row at its crossing of the tube-centre circle and
 // the tube g nearest to that crossing (candidates g - 1, g, g + 1).  False: it meets no row
 // or lies outside the rows' arc (no candidate tube), i.e. it misses the detector.
-template <typename R>
+template <typename R, bool NORM = false>
 __device__ __forceinline__ bool tubes_locate(const DetP<R>& D, const Ray<R>& n, int* row_out,
                                              int* g_out) {
   using M = Mth<R>;
   const R Rad = (R)D.radius;
   R sR;
-  if (!exit_cyl<R>(Rad, n, &sR)) return false;
+  if (!exit_cyl<R, NORM>(Rad, n, &sR)) return false;
   const R Px = n.x + sR * n.dx, Py = n.y + sR * n.dy, Pz = n.z + sR * n.dz;
   int row = -1;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    if (row < 0 && i < D.n_rows && M::fabs(Py - (R)D.row_y[i]) <= (R)D.half_len) row = i;
+    if (row < 0 && i < D.n_rows && M::le(M::fabs(Py - (R)D.row_y[i]), (R)D.half_len)) row = i;
   }
   if (row < 0) return false;
   const int tpp = D.tubes_per_pack;
@@ -1320,7 +1476,7 @@ __device__ __forceinline__ bool tubes_locate(const DetP<R>& D, const Ray<R>& n, 
 // The rest of the tube detector for a located packet: the first of the candidate tubes the
 // ray enters, the absorption point drawn from the truncated exponential of the 3He path
 // (u_det), pixel, time of flight and bin.
-template <typename R>
+template <typename R, bool NORM = false, int FORM = 0>
 __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W,
                                                const R* __restrict__ tu, const Ray<R>& n,
                                                R u_det, int row, int g) {
@@ -1339,26 +1495,28 @@ __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W
   const R y_hi = (R)D.row_y[row] + (R)D.half_len;
   int best = -1;
   R best_in = M::inf(), best_out = R(0);
-#pragma unroll
+  // FP64: one copy of the body (the FP64 kernels are bound by instruction fetch)
+#pragma unroll (sizeof(R) == 4 ? 3 : 1)
   for (int dc = -1; dc <= 1; ++dc) {
     const int c = g + dc;
     if (c < 0 || c >= n_tubes_row) continue;
     R s1, s2;
-    if (!tube_span<R>(Rad, tu[2 * c], tu[2 * c + 1], (R)D.tube_r, n, &s1, &s2)) continue;
+    if (!tube_span<R, NORM, FORM>(Rad, tu[2 * c], tu[2 * c + 1], (R)D.tube_r, n, &s1, &s2)) continue;
     R ys1, ys2;
-    if (n.dy == R(0)) {
+    if (M::is_zero(n.dy)) {
       if (!(n.y >= y_lo && n.y <= y_hi)) continue;
       ys1 = -M::inf();
       ys2 = M::inf();
     } else {
-      const R a = M::div(y_lo - n.y, n.dy), b = M::div(y_hi - n.y, n.dy);
+      const typename M::Rcp ry = M::rcp(n.dy);
+      const R a = M::divr(y_lo - n.y, ry), b = M::divr(y_hi - n.y, ry);
       ys1 = M::fmin(a, b);
       ys2 = M::fmax(a, b);
     }
     const R s_in = M::fmax(M::fmax(s1, ys1), R(0));
     const R s_out = M::fmin(s2, ys2);
-    if (!(s_out > s_in)) continue;
-    if (s_in < best_in) {
+    if (!M::lt(s_in, s_out)) continue;
+    if (M::lt(s_in, best_in)) {
       best = c;
       best_in = s_in;
       best_out = s_out;
@@ -1371,8 +1529,7 @@ __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W
   const R x = M::div(-M::log1p(-u_det * pabs), mu);
   const R s_abs = best_in + x;
   const R y_abs = n.y + s_abs * n.dy;
-  int j = (int)M::floor(M::div(y_abs - y_lo, (R)D.pix_len));
-  j = min(max(j, 0), D.pixels_per_tube - 1);
+  const int j = M::index_clamped(M::div(y_abs - y_lo, (R)D.pix_len), D.pixels_per_tube);
   const int pc = best / tpp, tc = best - pc * tpp;
   h.pixel = ((row_off + pc) * tpp + tc) * D.pixels_per_tube + j;
   h.tof.add(M::div(s_abs, n.speed));
@@ -1386,12 +1543,12 @@ __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W
 // Tube detector system (section 2.4.3, "Ray tracing in a detector system"): the packet's
 // crossing of the tube-centre circle picks the row and three candidate tubes; the first
 // tube the ray enters absorbs it.
-template <typename R>
+template <typename R, bool NORM, int FORM>
 __device__ __forceinline__ Hit<R> detect_tubes(const DetP<R>& D, const TofWin& W,
                                                const R* __restrict__ tu, const Ray<R>& n,
                                                R u_det) {
   int row = 0, g = 0;
-  if (!tubes_locate<R>(D, n, &row, &g)) {
+  if (!tubes_locate<R, NORM>(D, n, &row, &g)) {
     Hit<R> h;
     h.bin = -1;
     h.pixel = -1;
@@ -1400,15 +1557,22 @@ __device__ __forceinline__ Hit<R> detect_tubes(const DetP<R>& D, const TofWin& W
     h.pabs = R(0);
     return h;
   }
-  return tubes_absorb<R>(D, W, tu, n, u_det, row, g);
+  return tubes_absorb<R, NORM, FORM>(D, W, tu, n, u_det, row, g);
 }
 
-template <typename R, int DET, class Rng>
+// FP32 rounding of the detector trace.  The compiler's choice of fused multiply-adds differs from
+// kernel to kernel and with the code around; where a kernel's packets are detected in the same
+// block they are loaded in, it would have changed the detected weights of grazing chords by up
+// to 1e-4 of themselves.  The two expressions concerned are therefore written out:
+// NORM: the direction's squared horizontal length, fma(dz, dz, dx dx) (Mth::norm2);
+// FORM: r^2 - cr^2/a of a tube's chord, 1: fma(r, r, -(cr^2/a)), 2: fma(-cr^2, 1/a, r^2), 0: as the
+// compiler has it.
+template <typename R, int DET, bool NORM = false, int FORM = 0, class Rng>
 __device__ __forceinline__ Hit<R> detect(const DetP<R>& D, const TofWin& W, const R* tu,
                                          const Rng& rng, int order, const Ray<R>& n) {
-  if (DET == MCV_DET_SURFACE) return detect_surface<R>(D, W, n);
+  if (DET == MCV_DET_SURFACE) return detect_surface<R, NORM>(D, W, n);
   const R u = rng.template first<R>(order, 3);
-  return detect_tubes<R>(D, W, tu, n, u);
+  return detect_tubes<R, NORM, FORM>(D, W, tu, n, u);
 }
 
 // ---- tallies ---------------------------------------------------------------------------

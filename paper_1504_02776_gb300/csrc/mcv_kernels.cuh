@@ -48,7 +48,6 @@ struct LaunchOutT {
   static __device__ __forceinline__ double* tallies(const TraceArgs& A) { return A.tallies; }
   static __device__ __forceinline__ const EvSink& events(const TraceArgs& A) { return A.ev; }
 };
-using LaunchOut = LaunchOutT<true>;
 
 // one thread's running tallies: beam stop, detected and out-of-window weights, counts
 template <typename R>
@@ -57,22 +56,12 @@ struct Tally {
   Counts cnt;
 };
 
-// the tallies held in registers
-template <typename R>
-struct RegTally {
-  Tally<R> t;
-  __device__ __forceinline__ Tally<R>& get() { return t; }
-};
-
-// Forward policy: packets go to the packet slots and/or through the detector into the
-// histogram; order-0 packets go to the beam stop.  Out: where the histogram and tallies of
-// the simulation being traced are (read where used, so they hold no registers).  Store:
-// where the thread's running tallies are kept.
-template <typename R, int DET, class Out = LaunchOut, class Store = RegTally<R>>
+// Forward policy of the unfused path (trace_kernel): packets go to the packet slots and/or
+// through the detector into the histogram; order-0 packets go to the beam stop.
+template <typename R, int DET>
 struct Forward {
   static constexpr bool kWantsGs = false;
-  static constexpr bool kMeetingOnly = false;
-  Store store;
+  Tally<R> t;
   int err = 0;
 
   __device__ __forceinline__ void start(const Lane<R>&) {}
@@ -80,8 +69,7 @@ struct Forward {
   template <class Rng>
   __device__ __forceinline__ void emit(const TraceArgs& A, const R* tu, const Rng& rng,
                                        const Lane<R>& L, R we, R, R, R len_tot) {
-    Tally<R>& t = store.get();
-    if (L.o == 0 && len_tot > R(0)) t.cnt.nhit++;
+    if (L.o == 0 && Mth<R>::positive(len_tot)) t.cnt.nhit++;
     if (A.pk_order) store_slot<R>(A, L.idx * (Sof<R>(A).max_orders + 1) + L.o, L.n, we, L.nid, L.o);
     if (L.o == 0) {
       t.bs.add(we);
@@ -96,39 +84,13 @@ struct Forward {
 
   // a packet's detector result into the histogram and the tallies
   __device__ __forceinline__ void record(const TraceArgs& A, const Hit<R>& h) {
-    Tally<R>& t = store.get();
-    if constexpr (Out::kEvents) {
-      if (h.pixel >= 0 && Out::events(A).count)
-        append_event(Out::events(A), h.pixel, h.tof.value(), (double)h.w_det);
-    }
-    // Equal bins among the lanes recording together (a detector batch) are summed in the
-    // group's lowest lane and added with one FP64 atomic: fewer atomics on the bins that
-    // collect many events (the elastic line; low incident energies concentrate more).
-    const bool valid = h.bin >= 0 && h.bin < Dof<R>(A).n_bins;
-    const unsigned act = __activemask();
-    const int lane = threadIdx.x & 31;
-    const long long key = valid ? (long long)h.bin : -1ll - lane;
-    const unsigned peers = __match_any_sync(act, key);
-    if (valid) {
-      double* hist = Out::hist(A);
-      const double v = (double)h.w_det;
-      if (peers == (1u << lane)) {
-        if (hist) atomicAdd(hist + h.bin, v);
-      } else {
-        const int leader = __ffs(peers) - 1;
-        double sum = 0.0;
-        for (unsigned m = peers; m; m &= m - 1) {
-          const double x = __shfl_sync(peers, v, __ffs(m) - 1);
-          sum += x;
-        }
-        if (hist && lane == leader) atomicAdd(hist + h.bin, sum);
-      }
-    }
+    if (h.pixel >= 0 && A.ev.count) append_event(A.ev, h.pixel, h.tof.value(), (double)h.w_det);
     if (h.bin >= 0) {
       if (h.bin >= Dof<R>(A).n_bins) {
         err = 1;
         return;
       }
+      if (A.hist) atomicAdd(A.hist + h.bin, (double)h.w_det);
       t.det.add(h.w_det);
       t.cnt.ndet++;
     } else if (h.bin == -2) {
@@ -138,13 +100,6 @@ struct Forward {
       t.cnt.nmiss++;
     }
   }
-
-  // the beam stop's share of a packet of order 0, and an incident neutron meeting the sample
-  __device__ __forceinline__ void beam_stop(R w) { store.get().bs.add(w); }
-  // a packet that misses the detector system
-  __device__ __forceinline__ void missed() { store.get().cnt.nmiss++; }
-  __device__ __forceinline__ void hit() { store.get().cnt.nhit++; }
-  __device__ __forceinline__ void emitted() { store.get().cnt.nemit++; }
 
   __device__ __forceinline__ void scatter(const TraceArgs&, const Lane<R>&, int, R,
                                           const Scatter<R>&, R, R) {}
@@ -158,10 +113,8 @@ struct Forward {
     }
   }
 
-  // the warp's tallies into `tallies`; the accumulators start again from zero
   __device__ __forceinline__ void flush(const TraceArgs& A, int lane) {
-    double* tallies = Out::tallies(A);
-    Tally<R>& t = store.get();
+    double* tallies = A.tallies;
     if (tallies) {
       const double v_bs = warp_sum(t.bs.value());
       const double v_det = warp_sum(t.det.value());
@@ -181,7 +134,6 @@ struct Forward {
       }
     }
     if (__any_sync(0xffffffffu, err != 0) && lane == 0 && A.err) atomicOr(A.err, 1);
-    t = Tally<R>();
   }
 };
 
@@ -195,34 +147,157 @@ struct Forward {
 //             system and histograms it.
 // The per-neutron arithmetic is the chain step's and the detector's: only the order in
 // which lanes do the work changes, which keeps the lanes of a warp busy on the same code.
-constexpr int kWarps = kThreads / 32;
+//
+// Block size: one block per SM that fills it -- 640 threads in FP32 (20 warps at 96
+// registers), 384 in FP64 (12 warps at 168).  The kernels are bound by instruction fetch and
+// latency; against five blocks of 128 threads the one block measured 5.80 -> 5.12 ms (FP32
+// powder, 1e8 neutrons; two blocks of 320: 5.63; 576 threads: 6.05; 768 at 80 registers:
+// 6.83) and 1.60 -> 1.36 ms (vanadium-like powder, 1e7); in FP64, against three blocks of 128,
+// 5.04 -> 4.98 ms (5e6).  Shared memory below 164 KB leaves the L1 cache more room for the
+// kernels' tables.
+// Keeping the warps of a block in step with a barrier per round of the stages, so that they
+// fetch the same code together, cost more than it gave in FP32 (5.12 -> 6.88 ms).
+template <typename R>
+struct WaveCfg {
+  static constexpr int threads = sizeof(R) == 4 ? 640 : 384;
+  static constexpr int warps = threads / 32;
+};
 constexpr int kQueue = 64;  // per-warp queue capacity (at most 63 entries are ever held)
 
+// Queue entries hold a neutron's index in its simulation (below 2^40), not its 64-bit id.
 template <typename R>
-struct QNeutron {  // an incident neutron that meets the sample
-  R x, y, z, dx, dy, dz, speed;
+struct QNeutron {  // an incident neutron that meets the sample, at the start plane
+  R x, y, dx, dy, dz, speed;
   Tof<R> t;
-  int64_t nid;
+  uint32_t i_lo, i_hi;
 };
 
 template <typename R>
 struct QPacket {  // a transmitted packet of order >= 1 on its way to the detector
   R x, y, z, dx, dy, dz, speed, w;
   Tof<R> t;
-  int64_t nid;
-  int order;
-  int16_t row, g;  // located packets (FP64 tube detector): row, tube nearest to the crossing
+  uint32_t i_lo, i_hi_order;  // order in the low 8 bits
+};
+template <>
+struct QPacket<double> {
+  double x, y, z, dx, dy, dz, speed, w;
+  Tof<double> t;
+  uint32_t i_lo, i_hi_order;
+  int16_t row, g;  // located packets (tube detector): row, tube nearest to the crossing
+};
+
+// A footprint that may lead into the sample: its random words; the index's high bits in the
+// low bits of b, which no uniform uses.
+struct QFoot {
+  uint32_t a, b, c, d, i_lo;
 };
 
 template <typename R>
-struct QFoot {  // a footprint that may lead into the sample
-  R x, y;
-  int64_t nid;
+constexpr size_t queue_bytes() {  // of one warp
+  return (size_t)kQueue * (sizeof(QNeutron<R>) + sizeof(QPacket<R>) + sizeof(QFoot));
+}
+
+// The source stage's queues of one warp.
+template <typename R>
+struct SourceQueues {
+  QNeutron<R>* hq;
+  QFoot* fq;
+  int hq_n, fq_n;
 };
 
-template <typename R>
-constexpr size_t wave_smem_bytes() {
-  return (size_t)kWarps * kQueue * (sizeof(QNeutron<R>) + sizeof(QPacket<R>) + sizeof(QFoot<R>));
+// Source stage: queues neutrons until `need` are waiting or the ids run out.  Footprints
+// first, 32 new ids at a time: a neutron whose footprint cannot lead into the sample only adds
+// its weight, 1, to the beam stop; the others are queued.  Then 32 queued footprints at a time
+// get their divergence and, where they meet the sample, their energy: those are queued for the
+// sample stage, the rest add to the beam stop.  (Misses need no energy: the footprint bounds
+// are set only when every energy draw is positive.)  DROP: neutrons lighter than min_prob are
+// dropped here.  Returns the neutrons of weight 1 that miss the sample, the same in every lane.
+template <typename R, int NS, bool DROP, class Job, class Src>
+__device__ __forceinline__ uint32_t source_stage(const TraceArgs& A, const Job& job, int need,
+                                                 int64_t& next, int64_t& hi, Src& src,
+                                                 SourceQueues<R>& q) {
+  const SampleP<R>& S = job.S();
+  const unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  uint32_t missed = 0;
+  while (q.hq_n < need && (q.fq_n > 0 || next < hi || src.more(&next, &hi))) {
+    if (q.fq_n < 32 && (next < hi || src.more(&next, &hi))) {
+      const int64_t i = next + lane;
+      bool maybe = false;
+      Words w;
+      if (i < hi) {
+        w = job.rng(job.first_id() + i).words(-1, 1);
+        maybe = !footprint_misses<R>(job.B(), w);
+      }
+      const unsigned mm = __ballot_sync(kFull, maybe);
+      if (maybe)
+        q.fq[q.fq_n + __popc(mm & lt_mask)] =
+            QFoot{w.a, (w.b & ~0x7ffu) | (uint32_t)((uint64_t)i >> 32), w.c, w.d, (uint32_t)i};
+      q.fq_n += __popc(mm);
+      missed += (uint32_t)min((int64_t)32, hi - next) - __popc(mm);
+      next += 32;
+      __syncwarp();
+      continue;
+    }
+    const int take = q.fq_n < 32 ? q.fq_n : 32;
+    bool hit = false, miss = false;
+    Ray<R> nr;
+    uint32_t i_lo = 0, i_hi = 0;
+    if (lane < take) {
+      const QFoot f = q.fq[q.fq_n - take + lane];
+      i_lo = f.i_lo;
+      i_hi = f.b & 0x7ffu;
+      beam_footprint<R>(job.B(), Words{f.a, f.b, f.c, f.d}, &nr);
+    }
+    q.fq_n -= take;
+    __syncwarp();
+    if (lane < take) {
+      const auto rng = job.rng(job.first_id() + (int64_t)(((uint64_t)i_hi << 32) | i_lo));
+      R aux;
+      beam_divergence(job.B(), rng, &nr, &aux);
+      Seg<R> seg[2 * NS];
+      const bool meets = assembly_segs<R, NS>(S, nr, seg) > 0;
+      const bool ok = (meets || !job.B().energy_positive) ? beam_energy(job.B(), rng, aux, &nr)
+                                                          : true;
+      hit = ok && meets;
+      miss = ok && !meets;
+      if (DROP) hit = hit && !(nr.w < S.min_prob) && !(A.stop_on_zero && nr.w == R(0));
+    }
+    const unsigned hm = __ballot_sync(kFull, hit);
+    missed += __popc(__ballot_sync(kFull, miss));
+    if (hit) {
+      QNeutron<R>& e = q.hq[q.hq_n + __popc(hm & lt_mask)];
+      e.x = nr.x;
+      e.y = nr.y;
+      e.dx = nr.dx;
+      e.dy = nr.dy;
+      e.dz = nr.dz;
+      e.speed = nr.speed;
+      e.t = nr.t;
+      e.i_lo = i_lo;
+      e.i_hi = i_hi;
+    }
+    q.hq_n += __popc(hm);
+    __syncwarp();
+  }
+  // a neutron of weight 1 counts at the beam stop unless it is lighter than min_prob
+  return R(1) < S.min_prob ? 0u : missed;
+}
+
+// a queued neutron as a packet of order 0; returns its id
+template <typename R, class Job>
+__device__ __forceinline__ int64_t take_neutron(const Job& job, const QNeutron<R>& q, Ray<R>* n) {
+  n->x = q.x;
+  n->y = q.y;
+  n->z = -job.B().z0;
+  n->dx = q.dx;
+  n->dy = q.dy;
+  n->dz = q.dz;
+  n->speed = q.speed;
+  n->t = q.t;
+  n->w = R(1);
+  return job.first_id() + (int64_t)(((uint64_t)q.i_hi << 32) | q.i_lo);
 }
 
 extern __shared__ __align__(16) unsigned char g_wave_smem[];
@@ -248,34 +323,42 @@ struct BatchWarp {
   int home, v;
 };
 
-// Dynamic shared memory of the wave kernels: the warp queues, [the warps' batch slots,] and
-// every thread's running tallies (kept there rather than in registers).
-template <typename R>
-struct SmemTally {
-  size_t off;  // byte offset of the tallies in the dynamic shared memory
-  __device__ __forceinline__ Tally<R>& get() {
-    return reinterpret_cast<Tally<R>*>(g_wave_smem + off)[threadIdx.x];
-  }
+// A warp's counts, updated by its lane 0.
+struct WarpCounts {
+  uint32_t beam, hit, emit, miss, det, over;
 };
 
+// a thread's weight sums
 template <typename R>
-constexpr size_t wave_kernel_smem_bytes() {
-  return wave_smem_bytes<R>() + (size_t)kThreads * sizeof(Tally<R>);
-}
+struct WaveSums {
+  Acc<R> bs, det, over;
+};
 
+// Dynamic shared memory of the wave kernels: the warp queues, [the warps' batch slots,] every
+// thread's weight sums and every warp's counts (kept there rather than in registers), and the
+// directions of the tubes of a row.
 template <typename R>
-constexpr size_t batch_tally_offset() {
-  return wave_smem_bytes<R>() + (size_t)kWarps * sizeof(BatchWarp<R>);
+constexpr size_t wave_sums_offset(bool batch) {
+  return ((size_t)WaveCfg<R>::warps * (queue_bytes<R>() + (batch ? sizeof(BatchWarp<R>) : 0)) + 15) /
+         16 * 16;
 }
-
 template <typename R>
-constexpr size_t batch_smem_bytes() {
-  return batch_tally_offset<R>() + (size_t)kThreads * sizeof(Tally<R>);
+constexpr size_t wave_counts_offset(bool batch) {
+  return wave_sums_offset<R>(batch) + (size_t)WaveCfg<R>::threads * sizeof(WaveSums<R>);
+}
+template <typename R>
+constexpr size_t wave_tubes_offset(bool batch) {
+  return (wave_counts_offset<R>(batch) + WaveCfg<R>::warps * sizeof(WarpCounts) + 15) / 16 * 16;
+}
+template <typename R>
+size_t wave_smem_bytes(bool batch, int max_tubes_row) {
+  return wave_tubes_offset<R>(batch) + (size_t)2 * max_tubes_row * sizeof(R);
 }
 
 template <typename R>
 __device__ __forceinline__ BatchWarp<R>& batch_warp() {
-  return reinterpret_cast<BatchWarp<R>*>(g_wave_smem + wave_smem_bytes<R>())[threadIdx.x >> 5];
+  return reinterpret_cast<BatchWarp<R>*>(g_wave_smem + (size_t)WaveCfg<R>::warps *
+                                                           queue_bytes<R>())[threadIdx.x >> 5];
 }
 
 // further items of the simulation in the warp's slot, from its work queue
@@ -336,9 +419,105 @@ struct SlotJob {
   __device__ __forceinline__ int64_t first_id() const { return batch_warp<R>().sim.first_id; }
 };
 
+// Where the waves' results go: the histogram, the event list, the weight sums and counts.
+// Out: where the simulation's histogram and tallies are (read where used, so they hold no
+// registers).
+template <typename R, class Out, bool BATCH>
+struct WaveSink {
+  static constexpr bool kWantsGs = false;
+  int err = 0;
+
+  __device__ __forceinline__ WaveSums<R>& sums() {
+    return reinterpret_cast<WaveSums<R>*>(g_wave_smem + wave_sums_offset<R>(BATCH))[threadIdx.x];
+  }
+  __device__ __forceinline__ WarpCounts& counts() {
+    return reinterpret_cast<WarpCounts*>(g_wave_smem + wave_counts_offset<R>(BATCH))[threadIdx.x >> 5];
+  }
+  __device__ __forceinline__ void clear_all() {
+    sums() = WaveSums<R>();
+    if ((threadIdx.x & 31) == 0) counts() = WarpCounts{0, 0, 0, 0, 0, 0};
+    __syncwarp();
+  }
+
+  // The detector results of a batch of packets (`have`: this lane holds one) into the
+  // histogram and the tallies; called by the whole warp.
+  __device__ __forceinline__ void record(const TraceArgs& A, bool have, const Hit<R>& h) {
+    const unsigned kFull = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    if constexpr (Out::kEvents) {
+      if (have && h.pixel >= 0 && Out::events(A).count)
+        append_event(Out::events(A), h.pixel, h.tof.value(), (double)h.w_det);
+    }
+    const bool valid = have && h.bin >= 0 && h.bin < Dof<R>(A).n_bins;
+    const bool late = have && h.bin == -2;
+    if (have && h.bin >= Dof<R>(A).n_bins) err = 1;
+    const unsigned m_in = __ballot_sync(kFull, valid), m_over = __ballot_sync(kFull, late);
+    const unsigned m_miss = __ballot_sync(kFull, have && h.bin == -1);
+    if (lane == 0) {
+      WarpCounts& c = counts();
+      c.det += __popc(m_in);
+      c.over += __popc(m_over);
+      c.miss += __popc(m_miss);
+    }
+    // Equal bins among the lanes recording together are summed in the group's lowest lane and
+    // added with one FP64 atomic: fewer atomics on the bins that collect many events (the
+    // elastic line; low incident energies concentrate more).
+    if (valid) {
+      sums().det.add(h.w_det);
+      const unsigned peers = __match_any_sync(m_in, (long long)h.bin);
+      double* hist = Out::hist(A);
+      const double v = (double)h.w_det;
+      if (peers == (1u << lane)) {
+        if (hist) atomicAdd(hist + h.bin, v);
+      } else {
+        const int leader = __ffs(peers) - 1;
+        double sum = 0.0;
+        for (unsigned m = peers; m; m &= m - 1) {
+          const double x = __shfl_sync(peers, v, __ffs(m) - 1);
+          sum += x;
+        }
+        if (hist && lane == leader) atomicAdd(hist + h.bin, sum);
+      }
+    }
+    if (late) sums().over.add(h.w_det);
+    __syncwarp();
+  }
+
+  __device__ __forceinline__ void scatter(const TraceArgs&, const Lane<R>&, int, R,
+                                          const Scatter<R>&, R, R) {}
+  __device__ __forceinline__ void clear(const TraceArgs&, int64_t, int) {}
+
+  // the warp's sums and counts into the simulation's tallies; they start again from zero
+  __device__ __forceinline__ void flush(const TraceArgs& A, int lane) {
+    double* tallies = Out::tallies(A);
+    __syncwarp();
+    if (tallies) {
+      WaveSums<R>& t = sums();
+      const double v_bs = warp_sum(t.bs.value());
+      const double v_det = warp_sum(t.det.value());
+      const double v_over = warp_sum(t.over.value());
+      if (lane == 0) {
+        const WarpCounts& c = counts();
+        atomicAdd(tallies + MCV_T_BEAMSTOP, v_bs + (double)c.beam);
+        atomicAdd(tallies + MCV_T_WDET, v_det);
+        atomicAdd(tallies + MCV_T_WOVER, v_over);
+        atomicAdd(tallies + MCV_T_NDET, (double)c.det);
+        atomicAdd(tallies + MCV_T_NOVER, (double)c.over);
+        atomicAdd(tallies + MCV_T_NMISS, (double)c.miss);
+        atomicAdd(tallies + MCV_T_NHIT, (double)c.hit);
+        atomicAdd(tallies + MCV_T_NEMIT, (double)c.emit);
+      }
+    }
+    if (__any_sync(0xffffffffu, err != 0) && lane == 0 && A.err) atomicOr(A.err, 1);
+    __syncwarp();
+    clear_all();
+  }
+};
+
 // The waves of one warp over neutron ids first_id + [lo, hi) of one simulation, and over
 // every further range `src` hands out for it.  Returns with both queues empty.
-template <typename R, int NS, int DET, int KS, class Job, class Src, class P>
+// FORM: see detect().
+template <typename R, int NS, int DET, int KS, int FORM, class Job, class Src, class P>
 __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, int64_t lo,
                                           int64_t hi, const R* tu, P& pol, Src& src) {
   const SampleP<R>& S = job.S();
@@ -347,14 +526,14 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
-  QNeutron<R>* hq = reinterpret_cast<QNeutron<R>*>(g_wave_smem) + wib * kQueue;
-  QPacket<R>* dq = reinterpret_cast<QPacket<R>*>(g_wave_smem + (size_t)kWarps * kQueue *
-                                                   sizeof(QNeutron<R>)) + wib * kQueue;
-  QFoot<R>* fq = reinterpret_cast<QFoot<R>*>(
-                     g_wave_smem + (size_t)kWarps * kQueue * (sizeof(QNeutron<R>) + sizeof(QPacket<R>))) +
-                 wib * kQueue;
+  unsigned char* mine = g_wave_smem + (size_t)wib * queue_bytes<R>();
+  QPacket<R>* dq = reinterpret_cast<QPacket<R>*>(mine);
+  SourceQueues<R> q;
+  q.hq = reinterpret_cast<QNeutron<R>*>(mine + kQueue * sizeof(QPacket<R>));
+  q.fq = reinterpret_cast<QFoot*>(mine + kQueue * (sizeof(QPacket<R>) + sizeof(QNeutron<R>)));
+  q.hq_n = q.fq_n = 0;
   int64_t next = lo;
-  int hq_n = 0, dq_n = 0, fq_n = 0;
+  int dq_n = 0;
   Lane<R> L;
   L.active = false;
   L.o = 0;
@@ -363,105 +542,18 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
   for (;;) {
     const unsigned idle = __ballot_sync(kFull, !L.active);
     const int n_idle = __popc(idle);
-    // ---- source stage.  Footprints first, 32 new ids at a time: a neutron whose footprint
-    // cannot lead into the sample only adds its weight to the beam stop; the others are
-    // queued.  Then 32 queued footprints at a time get their divergence and, where they meet
-    // the sample, their energy: those are queued for the sample stage, the rest add to the
-    // beam stop.  (Misses need no energy: BeamP::x_safe is finite only when every energy
-    // draw is positive.)
-    while (hq_n < n_idle && (fq_n > 0 || next < hi || src.more(&next, &hi))) {
-      if (fq_n < 32 && (next < hi || src.more(&next, &hi))) {
-        const int64_t i = next + lane;
-        bool maybe = false;
-        Ray<R> nr;
-        int64_t nid = 0;
-        if (i < hi) {
-          nid = job.first_id() + i;
-          const auto rng = job.rng(nid);
-          beam_footprint(job.B(), rng, &nr);
-          if (!surely_misses<R>(job.B(), nr))
-            maybe = true;
-          else if (!(nr.w < S.min_prob) && !(A.stop_on_zero && nr.w == R(0)))
-            pol.beam_stop(nr.w * Mth<R>::exp(R(0)));  // order-0 packet, no material ahead
-        }
-        const unsigned mm = __ballot_sync(kFull, maybe);
-        if (maybe) {
-          QFoot<R>& f = fq[fq_n + __popc(mm & lt_mask)];
-          f.x = nr.x;
-          f.y = nr.y;
-          f.nid = nid;
-        }
-        fq_n += __popc(mm);
-        next += 32;
-        __syncwarp();
-        continue;
-      }
-      const int take_f = fq_n < 32 ? fq_n : 32;
-      bool hit = false;
-      Ray<R> nr;
-      int64_t nid = 0;
-      if (lane < take_f) {
-        const QFoot<R>& f = fq[fq_n - take_f + lane];
-        nid = f.nid;
-        nr.x = f.x;
-        nr.y = f.y;
-        nr.z = -job.B().z0;
-        nr.w = R(1);
-      }
-      fq_n -= take_f;
-      __syncwarp();
-      if (lane < take_f) {
-        const auto rng = job.rng(nid);
-        R aux;
-        beam_divergence(job.B(), rng, &nr, &aux);
-        Seg<R> seg[2 * NS];
-        const bool meets = assembly_segs<R, NS>(S, nr, seg) > 0;
-        bool ok = (meets || !job.B().energy_positive) ? beam_energy(job.B(), rng, aux, &nr)
-                                                      : true;
-        ok = ok && !(nr.w < S.min_prob) && !(A.stop_on_zero && nr.w == R(0));
-        if (ok) {
-          if (meets)
-            hit = true;
-          else
-            pol.beam_stop(nr.w * Mth<R>::exp(R(0)));  // order-0 packet, no material ahead
-        }
-      }
-      const unsigned hm = __ballot_sync(kFull, hit);
-      if (hit) {
-        QNeutron<R>& q = hq[hq_n + __popc(hm & lt_mask)];
-        q.x = nr.x;
-        q.y = nr.y;
-        q.z = nr.z;
-        q.dx = nr.dx;
-        q.dy = nr.dy;
-        q.dz = nr.dz;
-        q.speed = nr.speed;
-        q.t = nr.t;
-        q.nid = nid;
-      }
-      hq_n += __popc(hm);
-      __syncwarp();
-    }
-    const int take = min(n_idle, hq_n);
+    // ---- source stage
+    const uint32_t n_beam = source_stage<R, NS, true>(A, job, n_idle, next, hi, src, q);
+    const int take = min(n_idle, q.hq_n);
     if (!L.active) {
       const int r = __popc(idle & lt_mask);
       if (r < take) {
-        const QNeutron<R>& q = hq[hq_n - take + r];
-        L.n.x = q.x;
-        L.n.y = q.y;
-        L.n.z = q.z;
-        L.n.dx = q.dx;
-        L.n.dy = q.dy;
-        L.n.dz = q.dz;
-        L.n.speed = q.speed;
-        L.n.t = q.t;
-        L.n.w = R(1);
-        L.nid = q.nid;
+        L.nid = take_neutron<R>(job, q.hq[q.hq_n - take + r], &L.n);
         L.o = 0;
         L.active = true;
       }
     }
-    hq_n -= take;
+    q.hq_n -= take;
     __syncwarp();
     // ---- sample stage.  FP64: a transmitted packet of order >= 1 is first located on the
     // tube rows (row and candidate tubes) and only packets that can reach a tube are queued
@@ -471,28 +563,37 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
     constexpr bool kLocateEarly = DET == MCV_DET_TUBES && sizeof(R) == 8;
     StepState<R, NS> st;
     R we = R(0);
-    bool to_det = false;
+    bool to_det = false, missed = false, hit = false;
     int row = 0, g = 0;
     if (L.active) {
       we = step_segments<R, NS, false>(A, S, L, st);
       if (L.o == 0) {
-        pol.beam_stop(we);
-        if (st.len_tot > R(0)) pol.hit();
+        pol.sums().bs.add(we);
+        hit = Mth<R>::positive(st.len_tot);
+      } else if (DET == MCV_DET_TUBES && det_surely_misses<R>(D, L.n)) {
+        missed = true;
+      } else if constexpr (kLocateEarly) {
+        to_det = tubes_locate<R>(D, L.n, &row, &g);
+        missed = !to_det;
       } else {
-        pol.emitted();
-        if (DET == MCV_DET_TUBES && det_surely_misses<R>(D, L.n))
-          pol.missed();
-        else if (!kLocateEarly || tubes_locate<R>(D, L.n, &row, &g))
-          to_det = true;
-        else
-          pol.missed();
+        to_det = true;
       }
     }
-    const unsigned dm = __ballot_sync(kFull, to_det);
+    const unsigned dm = __ballot_sync(kFull, to_det), miss_m = __ballot_sync(kFull, missed);
+    const unsigned hit_m = __ballot_sync(kFull, hit);
+    if (lane == 0) {
+      WarpCounts& c = pol.counts();
+      c.beam += n_beam;
+      c.hit += __popc(hit_m);
+      c.emit += __popc(dm) + __popc(miss_m);
+      c.miss += __popc(miss_m);
+    }
     if (to_det) {
       QPacket<R>& p = dq[dq_n + __popc(dm & lt_mask)];
-      p.row = (int16_t)row;
-      p.g = (int16_t)g;
+      if constexpr (kLocateEarly) {
+        p.row = (int16_t)row;
+        p.g = (int16_t)g;
+      }
       p.x = L.n.x;
       p.y = L.n.y;
       p.z = L.n.z;
@@ -502,12 +603,13 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
       p.speed = L.n.speed;
       p.w = we;
       p.t = L.n.t;
-      p.nid = L.nid;
-      p.order = L.o;
+      const uint64_t i = (uint64_t)(L.nid - job.first_id());
+      p.i_lo = (uint32_t)i;
+      p.i_hi_order = ((uint32_t)(i >> 32) << 8) | (uint32_t)L.o;
     }
     dq_n += __popc(dm);
     if (L.active) {
-      if (L.o == S.max_orders || !(st.len_tot > R(0))) {
+      if (L.o == S.max_orders || !Mth<R>::positive(st.len_tot)) {
         L.active = false;
       } else {
         const auto rng = job.rng(L.nid);
@@ -518,17 +620,27 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
     // ---- detector stage: full batches now, the remainder once the range is done.  This is
     // the only place packets are detected, so a packet's arithmetic does not depend on the
     // batch it falls in (or on the launch shape).
-    bool done = !__any_sync(kFull, L.active) && next >= hi && hq_n == 0 && fq_n == 0;
+    bool done = !__any_sync(kFull, L.active) && next >= hi && q.hq_n == 0 && q.fq_n == 0;
     if (done) done = !src.more(&next, &hi);
     while (dq_n >= 32 || (done && dq_n > 0)) {
-      const int take = dq_n < 32 ? dq_n : 32;
+      const int take_d = dq_n < 32 ? dq_n : 32;
+      const bool have = lane < take_d;
+      Hit<R> h;
+      h.bin = -1;
+      h.pixel = -1;
+      h.w_det = R(0);
+      // The wide kernels load the packets in a block of their own: the compiler's choice of
+      // fused multiply-adds depends on the block, and the FP32 results on that choice.  (In
+      // one block, as the powder kernels have it, fewer registers spill: 4.93 -> 4.66 ms.)
       Ray<R> pe;
       int order = 0, row = 0, g = 0;
       int64_t nid = 0;
-      if (lane < take) {
-        const QPacket<R>& p = dq[dq_n - take + lane];
-        row = p.row;
-        g = p.g;
+      if (have) {
+        const QPacket<R>& p = dq[dq_n - take_d + lane];
+        if constexpr (kLocateEarly) {
+          row = p.row;
+          g = p.g;
+        }
         pe.x = p.x;
         pe.y = p.y;
         pe.z = p.z;
@@ -538,20 +650,20 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
         pe.speed = p.speed;
         pe.t = p.t;
         pe.w = p.w;
-        nid = p.nid;
-        order = p.order;
+        order = (int)(p.i_hi_order & 0xffu);
+        nid = job.first_id() + (int64_t)(((uint64_t)(p.i_hi_order >> 8) << 32) | p.i_lo);
+      }
+      if constexpr (KS != kKernelsPowder) __syncwarp();
+      if (have) {
+        const auto rng = job.rng(nid);
+        if constexpr (kLocateEarly)
+          h = tubes_absorb<R>(D, job.W(), tu, pe, rng.template first<R>(order, 3), row, g);
+        else
+          h = detect<R, DET, KS == kKernelsPowder, FORM>(D, job.W(), tu, rng, order, pe);
       }
       __syncwarp();
-      if (lane < take) {
-        const auto rng = job.rng(nid);
-        if (kLocateEarly) {
-          const R u = rng.template first<R>(order, 3);
-          pol.record(A, tubes_absorb<R>(D, job.W(), tu, pe, u, row, g));
-        } else {
-          pol.record(A, detect<R, DET>(D, job.W(), tu, rng, order, pe));
-        }
-      }
-      dq_n -= take;
+      pol.record(A, have, h);
+      dq_n -= take_d;
     }
     if (done) break;
   }
@@ -565,32 +677,20 @@ __global__ void __launch_bounds__(kThreads) trace_kernel(const __grid_constant__
   run_chain<R, NS, DET, KS, Forward<R, DET>>(A, tu, pol);
 }
 
-// resident blocks per SM the register allocation aims at (FP64 state needs more registers)
-#ifndef MCV_WAVE_BLOCKS_F32
-#define MCV_WAVE_BLOCKS_F32 5
-#endif
-#ifndef MCV_WAVE_BLOCKS_F64
-#define MCV_WAVE_BLOCKS_F64 3
-#endif
-template <typename R>
-struct WaveBlocks {
-  static constexpr int value = sizeof(R) == 4 ? MCV_WAVE_BLOCKS_F32 : MCV_WAVE_BLOCKS_F64;
-};
-
 template <typename R, int NS, int DET, int KS, bool EV>
-__global__ void __launch_bounds__(kThreads, WaveBlocks<R>::value)
+__global__ void __launch_bounds__(WaveCfg<R>::threads, 1)
     wave_kernel(const __grid_constant__ TraceArgs A) {
-  __shared__ R tu[2 * MCV_MAX_TUBES_PER_ROW];
+  R* tu = reinterpret_cast<R*>(g_wave_smem + wave_tubes_offset<R>(false));
   stage_tubes<R, DET>(A, tu);
-  Forward<R, DET, LaunchOutT<EV>, SmemTally<R>> pol{SmemTally<R>{wave_smem_bytes<R>()}};
-  pol.store.get() = Tally<R>();
+  WaveSink<R, LaunchOutT<EV>, false> pol;
+  pol.clear_all();
   // each warp owns one contiguous range of the launch's neutron ids
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t lo = (A.n * wid) / nw, hi = (A.n * (wid + 1)) / nw;
   NoMoreIds src;
   const ParamJob<R> job{A};
-  run_waves<R, NS, DET, KS>(A, job, lo, hi, tu, pol, src);
+  run_waves<R, NS, DET, KS, NS == 1 && KS == kKernelsPowder ? 1 : 2>(A, job, lo, hi, tu, pol, src);
   pol.flush(A, threadIdx.x & 31);
 }
 
@@ -605,9 +705,9 @@ __global__ void __launch_bounds__(kThreads, WaveBlocks<R>::value)
 // kernel's.
 // SS: every simulation has the batch's sample (A.Sf / A.Sd), kept in parameter space
 template <typename R, int NS, int DET, int KS, bool SS, bool EV>
-__global__ void __launch_bounds__(kThreads, WaveBlocks<R>::value)
+__global__ void __launch_bounds__(WaveCfg<R>::threads, 1)
     batch_wave_kernel(const __grid_constant__ TraceArgs A, const __grid_constant__ BatchArgs Q) {
-  __shared__ R tu[2 * MCV_MAX_TUBES_PER_ROW];
+  R* tu = reinterpret_cast<R*>(g_wave_smem + wave_tubes_offset<R>(true));
   stage_tubes<R, DET>(A, tu);
   const int lane = threadIdx.x & 31;
   {
@@ -629,8 +729,8 @@ __global__ void __launch_bounds__(kThreads, WaveBlocks<R>::value)
     }
     __syncwarp();
   }
-  Forward<R, DET, SlotOut<R, EV>, SmemTally<R>> pol{SmemTally<R>{batch_tally_offset<R>()}};
-  pol.store.get() = Tally<R>();
+  WaveSink<R, SlotOut<R, EV>, true> pol;
+  pol.clear_all();
   const SlotJob<R, SS> job{A};
   QueuedIds<R> src;
   for (;;) {
@@ -655,7 +755,7 @@ __global__ void __launch_bounds__(kThreads, WaveBlocks<R>::value)
     uint32_t* to = reinterpret_cast<uint32_t*>(&me.sim);
     for (int w = lane; w < (int)(sizeof(SimP<R>) / 4); w += 32) to[w] = from[w];
     __syncwarp();
-    run_waves<R, NS, DET, KS>(A, job, lo, hi, tu, pol, src);
+    run_waves<R, NS, DET, KS, 1>(A, job, lo, hi, tu, pol, src);
     pol.flush(A, lane);
   }
 }
@@ -784,9 +884,6 @@ __global__ void __launch_bounds__(kThreads) detect_kernel(const __grid_constant_
 template <typename R, int DET>
 struct Adjoint {
   static constexpr bool kWantsGs = true;
-  // a neutron that does not meet the sample only reaches the beam stop, which carries no
-  // gradient: its divergence and energy are not drawn
-  static constexpr bool kMeetingOnly = true;
   R a[kMaxOrders];   // scattering factor without the table value
   R s[kMaxOrders];   // table value (1 for kernels without a table)
   int e[kMaxOrders]; // table entry or -1
@@ -869,25 +966,22 @@ struct Adjoint {
   }
 };
 
-// Warp loop of a policy that keeps only the neutrons meeting the sample (the adjoint): the
-// source draws are compacted as in the waves -- footprints 32 new ids at a time, those that
-// may lead into the sample queued; then 32 queued footprints at a time get their direction
-// and, where they meet the sample, their energy, and are queued as neutrons -- and the lanes
-// without a neutron take queued ones, so that the chain steps run on full warps.  The
-// neutrons and their arithmetic are those of run_chain with make_beam_meeting.
+// Warp loop of a policy that keeps only the neutrons meeting the sample (the adjoint: the
+// others only reach the beam stop, which carries no gradient): the waves' source stage, and
+// the lanes without a neutron take queued ones, so that the chain steps run on full warps.
 template <typename R, int NS, int DET, int KS, class P>
 __device__ __forceinline__ void run_chain_meeting(const TraceArgs& A, const R* tu, P& pol,
-                                                  QNeutron<R>* hq, QFoot<R>* fq) {
+                                                  QNeutron<R>* hq, QFoot* fq) {
   const unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t lo = (A.n * wid) / nw, hi = (A.n * (wid + 1)) / nw;
-  const SampleP<R>& S = Sof<R>(A);
-  const BeamP<R>& Bm = Bof<R>(A);
-  int64_t next = lo;
-  int hq_n = 0, fq_n = 0;  // queued neutrons and footprints (each at most 63)
+  const int64_t lo = (A.n * wid) / nw;
+  int64_t hi = (A.n * (wid + 1)) / nw, next = lo;
+  const ParamJob<R> job{A};
+  NoMoreIds src;
+  SourceQueues<R> q{hq, fq, 0, 0};
   Lane<R> L;
   L.active = false;
   L.o = 0;
@@ -896,90 +990,19 @@ __device__ __forceinline__ void run_chain_meeting(const TraceArgs& A, const R* t
   for (;;) {
     const unsigned idle = __ballot_sync(kFull, !L.active);
     const int n_idle = __popc(idle);
-    while (hq_n < n_idle && (fq_n > 0 || next < hi)) {
-      if (fq_n < 32 && next < hi) {
-        const int64_t i = next + lane;
-        bool maybe = false;
-        Ray<R> nr;
-        int64_t nid = 0;
-        if (i < hi) {
-          nid = A.first_id + i;
-          const NeutronRng rng(A.keys, nid);
-          beam_footprint(Bm, rng, &nr);
-          maybe = !surely_misses<R>(Bm, nr);
-        }
-        const unsigned mm = __ballot_sync(kFull, maybe);
-        if (maybe) {
-          QFoot<R>& f = fq[fq_n + __popc(mm & lt_mask)];
-          f.x = nr.x;
-          f.y = nr.y;
-          f.nid = nid;
-        }
-        fq_n += __popc(mm);
-        next += 32;
-        __syncwarp();
-        continue;
-      }
-      const int take_f = fq_n < 32 ? fq_n : 32;
-      bool hit = false;
-      Ray<R> nr;
-      int64_t nid = 0;
-      if (lane < take_f) {
-        const QFoot<R>& f = fq[fq_n - take_f + lane];
-        nid = f.nid;
-        nr.x = f.x;
-        nr.y = f.y;
-        nr.z = -Bm.z0;
-        nr.w = R(1);
-      }
-      fq_n -= take_f;
-      __syncwarp();
-      if (lane < take_f) {
-        const NeutronRng rng(A.keys, nid);
-        R aux;
-        beam_divergence(Bm, rng, &nr, &aux);
-        Seg<R> seg[2 * NS];
-        if (assembly_segs<R, NS>(S, nr, seg) > 0 && beam_energy(Bm, rng, aux, &nr))
-          hit = !(nr.w < S.min_prob) && !(A.stop_on_zero && nr.w == R(0));
-      }
-      const unsigned hm = __ballot_sync(kFull, hit);
-      if (hit) {
-        QNeutron<R>& q = hq[hq_n + __popc(hm & lt_mask)];
-        q.x = nr.x;
-        q.y = nr.y;
-        q.z = nr.z;
-        q.dx = nr.dx;
-        q.dy = nr.dy;
-        q.dz = nr.dz;
-        q.speed = nr.speed;
-        q.t = nr.t;
-        q.nid = nid;
-      }
-      hq_n += __popc(hm);
-      __syncwarp();
-    }
-    const int take = min(n_idle, hq_n);
+    source_stage<R, NS, true>(A, job, n_idle, next, hi, src, q);
+    const int take = min(n_idle, q.hq_n);
     if (!L.active) {
       const int r = __popc(idle & lt_mask);
       if (r < take) {
-        const QNeutron<R>& q = hq[hq_n - take + r];
-        L.n.x = q.x;
-        L.n.y = q.y;
-        L.n.z = q.z;
-        L.n.dx = q.dx;
-        L.n.dy = q.dy;
-        L.n.dz = q.dz;
-        L.n.speed = q.speed;
-        L.n.t = q.t;
-        L.n.w = R(1);
-        L.nid = q.nid;
-        L.idx = q.nid - A.first_id;
+        L.nid = take_neutron<R>(job, q.hq[q.hq_n - take + r], &L.n);
+        L.idx = L.nid - A.first_id;
         L.o = 0;
         L.active = true;
         pol.start(L);
       }
     }
-    hq_n -= take;
+    q.hq_n -= take;
     __syncwarp();
     // no lane holds a neutron only once the queues are empty and the range is done
     if (!__any_sync(kFull, L.active)) break;
@@ -991,8 +1014,8 @@ __device__ __forceinline__ void run_chain_meeting(const TraceArgs& A, const R* t
 template <typename R, int NS, int DET, int KS>
 __global__ void __launch_bounds__(kThreads) adjoint_kernel(const __grid_constant__ TraceArgs A) {
   __shared__ R tu[2 * MCV_MAX_TUBES_PER_ROW];
-  __shared__ QNeutron<R> hq[kWarps * kQueue];
-  __shared__ QFoot<R> fq[kWarps * kQueue];
+  __shared__ QNeutron<R> hq[kThreads / 32 * kQueue];
+  __shared__ QFoot fq[kThreads / 32 * kQueue];
   stage_tubes<R, DET>(A, tu);
   Adjoint<R, DET> pol;
   const int wib = threadIdx.x >> 5;
@@ -1017,15 +1040,29 @@ cudaError_t launch_waves_ev(const TraceArgs& A, int det, int grid, cudaStream_t 
   return sizeof(R) == 4 ? launch_waves_ev_f32(A, det, grid, s) : launch_waves_ev_f64(A, det, grid, s);
 }
 
+template <typename R>
+const DetP<R>& Dof_host(const TraceArgs& A) {
+  if constexpr (sizeof(R) == 4)
+    return A.Df;
+  else
+    return A.Dd;
+}
+
+// the largest dynamic shared memory a wave kernel is launched with (the longest tube row)
+template <typename R>
+cudaError_t allow_wave_smem(const void* fn, bool batch) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)wave_smem_bytes<R>(batch, MCV_MAX_TUBES_PER_ROW));
+}
+
 template <typename R, int NS, int DET, int KS>
 cudaError_t launch_trace_k(const TraceArgs& A, int grid, cudaStream_t s) {
   if (DET != MCV_DET_NONE && uses_waves(A, DET)) {
     if (A.ev.count) return launch_waves_ev<R>(A, DET, grid, s);
-    const size_t smem = wave_kernel_smem_bytes<R>();
-    cudaError_t e = cudaFuncSetAttribute(wave_kernel<R, NS, DET, KS, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = wave_smem_bytes<R>(false, Dof_host<R>(A).max_tubes_row);
+    cudaError_t e = allow_wave_smem<R>((const void*)wave_kernel<R, NS, DET, KS, false>, false);
     if (e != cudaSuccess) return e;
-    wave_kernel<R, NS, DET, KS, false><<<grid, kThreads, smem, s>>>(A);
+    wave_kernel<R, NS, DET, KS, false><<<grid, WaveCfg<R>::threads, smem, s>>>(A);
   } else {
     trace_kernel<R, NS, DET, KS><<<grid, kThreads, 0, s>>>(A);
   }
@@ -1035,13 +1072,13 @@ cudaError_t launch_trace_k(const TraceArgs& A, int grid, cudaStream_t s) {
 // the waves with an event list, over the shapes (used by the _ev translation units)
 template <typename R, int NS, int KS>
 cudaError_t launch_waves_ev_k(const TraceArgs& A, int det, int grid, cudaStream_t s) {
-  const size_t smem = wave_kernel_smem_bytes<R>();
+  const size_t smem = wave_smem_bytes<R>(false, Dof_host<R>(A).max_tubes_row);
   const void* fn = det == MCV_DET_SURFACE ? (const void*)wave_kernel<R, NS, MCV_DET_SURFACE, KS, true>
                                           : (const void*)wave_kernel<R, NS, MCV_DET_TUBES, KS, true>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_wave_smem<R>(fn, false);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<TraceArgs*>(&A)};
-  return cudaLaunchKernel(fn, dim3(grid), dim3(kThreads), args, smem, s);
+  return cudaLaunchKernel(fn, dim3(grid), dim3(WaveCfg<R>::threads), args, smem, s);
 }
 
 template <typename R>
@@ -1099,12 +1136,12 @@ template <typename R>
 cudaError_t blocks_per_sm_t(int ns, int det, int bvk, int* blocks) {
   const void* fn = ns <= 1 ? trace_fn_ns<R, 1>(det, bvk) : (ns == 2 ? trace_fn_ns<R, 2>(det, bvk)
                                                                     : trace_fn_ns<R, 4>(det, bvk));
-  const size_t smem = det != MCV_DET_NONE ? wave_kernel_smem_bytes<R>() : 0;
-  if (smem) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kThreads, smem);
+  if (det == MCV_DET_NONE)
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kThreads, 0);
+  cudaError_t e = allow_wave_smem<R>(fn, false);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      blocks, fn, WaveCfg<R>::threads, wave_smem_bytes<R>(false, MCV_MAX_TUBES_PER_ROW));
 }
 
 // the batched kernel of a shape; its dynamic shared memory limit is set where its occupancy
@@ -1138,10 +1175,10 @@ const void* batch_fn_t(int ns, int det, int bvk, int ss) {
 template <typename R, bool EV>
 cudaError_t batch_blocks_per_sm_t(int ns, int det, int bvk, int ss, int* blocks) {
   const void* fn = batch_fn_t<R, EV>(ns, det, bvk, ss);
-  const size_t smem = batch_smem_bytes<R>();
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_wave_smem<R>(fn, true);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kThreads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      blocks, fn, WaveCfg<R>::threads, wave_smem_bytes<R>(true, MCV_MAX_TUBES_PER_ROW));
 }
 
 template <typename R, bool EV>
@@ -1149,7 +1186,8 @@ cudaError_t launch_batch_t(const TraceArgs& A, const BatchArgs& Q, int ns, int d
                            int ss, int grid, cudaStream_t s) {
   const void* fn = batch_fn_t<R, EV>(ns, det, bvk, ss);
   void* args[] = {const_cast<TraceArgs*>(&A), const_cast<BatchArgs*>(&Q)};
-  return cudaLaunchKernel(fn, dim3(grid), dim3(kThreads), args, batch_smem_bytes<R>(), s);
+  return cudaLaunchKernel(fn, dim3(grid), dim3(WaveCfg<R>::threads), args,
+                          wave_smem_bytes<R>(true, Dof_host<R>(A).max_tubes_row), s);
 }
 
 template <typename R>
@@ -1239,6 +1277,7 @@ cudaError_t launch_paper_t(const TraceArgs& A, int det, int grid, cudaStream_t s
   cudaError_t launch_trace_##SUFFIX(const TraceArgs& A, int det, int grid, cudaStream_t s) { \
     return launch_trace_t<R>(A, det, grid, s);                                              \
   }                                                                                         \
+  int wave_threads_##SUFFIX() { return WaveCfg<R>::threads; }                               \
   cudaError_t blocks_per_sm_##SUFFIX(int ns, int det, int bvk, int* blocks) {               \
     return blocks_per_sm_t<R>(ns, det, bvk, blocks);                                        \
   }

@@ -18,6 +18,8 @@ struct EventsArgs {
 };
 
 int trace_threads();
+// threads per block of the fused (waves) and batched kernels
+int wave_threads(int fp_mode);
 cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int* blocks);
 cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, int grid, cudaStream_t s);
 cudaError_t launch_beam(const TraceArgs& A, int fp_mode, int grid, cudaStream_t s);

@@ -80,19 +80,20 @@ __device__ __forceinline__ int tubes_absorb_multi(const DetP<R>& D, const TofWin
     R s1, s2;
     if (!tube_span<R>(Rad, tu[2 * c], tu[2 * c + 1], (R)D.tube_r, n, &s1, &s2)) continue;
     R ys1, ys2;
-    if (n.dy == R(0)) {
+    if (M::is_zero(n.dy)) {
       if (!(n.y >= y_lo && n.y <= y_hi)) continue;
       ys1 = -M::inf();
       ys2 = M::inf();
     } else {
-      const R a = M::div(y_lo - n.y, n.dy), b = M::div(y_hi - n.y, n.dy);
+      const typename M::Rcp ry = M::rcp(n.dy);
+      const R a = M::divr(y_lo - n.y, ry), b = M::divr(y_hi - n.y, ry);
       ys1 = M::fmin(a, b);
       ys2 = M::fmax(a, b);
     }
     const R a_in = M::fmax(M::fmax(s1, ys1), R(0)), a_out = M::fmin(s2, ys2);
-    if (!(a_out > a_in)) continue;
+    if (!M::lt(a_in, a_out)) continue;
     int at = m++;
-    while (at > 0 && s_in[at - 1] > a_in) {  // insertion by entry distance
+    while (at > 0 && M::lt(a_in, s_in[at - 1])) {  // insertion by entry distance
       tube[at] = tube[at - 1];
       s_in[at] = s_in[at - 1];
       s_out[at] = s_out[at - 1];
@@ -110,8 +111,7 @@ __device__ __forceinline__ int tubes_absorb_multi(const DetP<R>& D, const TofWin
     const R x = M::div(-M::log1p(-u[i] * pabs), mu);
     const R s_abs = s_in[i] + x;
     const R y_abs = n.y + s_abs * n.dy;
-    int j = (int)M::floor(M::div(y_abs - y_lo, (R)D.pix_len));
-    j = min(max(j, 0), D.pixels_per_tube - 1);
+    const int j = M::index_clamped(M::div(y_abs - y_lo, (R)D.pix_len), D.pixels_per_tube);
     const int pc = tube[i] / tpp, tc = tube[i] - pc * tpp;
     h[i].pixel = ((row_off + pc) * tpp + tc) * D.pixels_per_tube + j;
     h[i].tof = n.t;
@@ -172,7 +172,7 @@ constexpr int kPaperWarps = kPaperThreads / 32;
 template <typename R>
 constexpr size_t paper_smem_bytes() {
   return (size_t)kPaperWarps * kQueue *
-         (sizeof(QNeutron<R>) + sizeof(QFoot<R>) + sizeof(PaperDet<R>));
+         (sizeof(QNeutron<R>) + sizeof(QFoot) + sizeof(PaperDet<R>));
 }
 
 // a packet leaving the sample assembly
@@ -247,7 +247,7 @@ __device__ __forceinline__ int paper_interact1(const TraceArgs& A, const SampleP
   p.n.t.add(M::div(s, in.n.speed));
   p.n.w = in.n.w * sc.mu_s * len * M::exp(-mu * ell);
   p.s0 = R(0);
-  const int kk = (sc.nk == 2 && !(u_k * sc.ksig_sum < sc.ksig0)) ? 1 : 0;
+  const int kk = (sc.nk == 2 && !M::lt_nonneg(u_k * sc.ksig_sum, sc.ksig0)) ? 1 : 0;
   Scatter<R> out;
   if (!scatter_kernel<R, KS>(S, sc, kk, rng, 0, &p.n, &out, err)) return 2;
   p.n.w = p.n.w * out.factor;
@@ -280,7 +280,7 @@ __device__ __forceinline__ void paper_step(const TraceArgs& A, int64_t nid, Pape
   Seg<R> seg[2 * NS];
   const int ns = assembly_segs<R, NS>(S, cur.n, seg, cur.s0);
   if (cur.node == 1 && ns > 0) T.cnt.nhit++;
-  if (cur.n.w < S.min_prob) return;
+  if (Mth<R>::lt(cur.n.w, S.min_prob)) return;
   int j = -1;
   R a = R(0), b = R(0);
   if (jp >= 0) {  // path1 goes on: the scatterer's first segment ahead, if any
@@ -332,25 +332,25 @@ template <typename R, int NS, int DET, int KS>
 __global__ void __launch_bounds__(kPaperThreads) paper_kernel(const __grid_constant__ TraceArgs A) {
   __shared__ R tu[2 * MCV_MAX_TUBES_PER_ROW];
   const int wib = threadIdx.x >> 5;
-  QNeutron<R>* hq = reinterpret_cast<QNeutron<R>*>(g_wave_smem) + wib * kQueue;
-  QFoot<R>* fq = reinterpret_cast<QFoot<R>*>(
-                     g_wave_smem + (size_t)kPaperWarps * kQueue * sizeof(QNeutron<R>)) +
-                 wib * kQueue;
-  PaperDet<R>* dq = reinterpret_cast<PaperDet<R>*>(
-                        g_wave_smem + (size_t)kPaperWarps * kQueue *
-                                          (sizeof(QNeutron<R>) + sizeof(QFoot<R>))) +
-                    wib * kQueue;
+  PaperDet<R>* dq = reinterpret_cast<PaperDet<R>*>(g_wave_smem) + wib * kQueue;
+  unsigned char* after = g_wave_smem + (size_t)kPaperWarps * kQueue * sizeof(PaperDet<R>);
+  SourceQueues<R> q;
+  q.hq = reinterpret_cast<QNeutron<R>*>(after) + wib * kQueue;
+  q.fq = reinterpret_cast<QFoot*>(after + (size_t)kPaperWarps * kQueue * sizeof(QNeutron<R>)) +
+         wib * kQueue;
+  q.hq_n = q.fq_n = 0;
   stage_tubes<R, DET>(A, tu);
   const SampleP<R>& S = Sof<R>(A);
-  const BeamP<R>& Bm = Bof<R>(A);
+  const ParamJob<R> job{A};
+  NoMoreIds src;
   const unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t lo = (A.n * wid) / nw, hi = (A.n * (wid + 1)) / nw;
-  int64_t next = lo;
-  int hq_n = 0, fq_n = 0, dq_n = 0;  // queued neutrons, footprints, packets (each <= 63)
+  int64_t next = (A.n * wid) / nw, hi = (A.n * (wid + 1)) / nw;
+  int dq_n = 0;  // queued packets (at most 63)
+  uint64_t n_beam = 0;  // neutrons that miss the sample, the same in every lane
   PaperTally<R> T;
   PaperPk<R> stack[kPaperStack];
   PaperPk<R> cur;
@@ -360,102 +360,22 @@ __global__ void __launch_bounds__(kPaperThreads) paper_kernel(const __grid_const
   for (;;) {
     const unsigned idle = __ballot_sync(kFull, !busy);
     const int n_idle = __popc(idle);
-    while (hq_n < n_idle && (fq_n > 0 || next < hi)) {
-      if (fq_n < 32 && next < hi) {
-        const int64_t i = next + lane;
-        bool maybe = false;
-        Ray<R> nr;
-        int64_t id = 0;
-        if (i < hi) {
-          id = A.first_id + i;
-          const NeutronRng rng(A.keys, id);
-          beam_footprint(Bm, rng, &nr);
-          if (!surely_misses<R>(Bm, nr))
-            maybe = true;
-          else if (!(nr.w < S.min_prob))
-            T.bs.add(nr.w);  // order-0 packet, no material ahead
-        }
-        const unsigned mm = __ballot_sync(kFull, maybe);
-        if (maybe) {
-          QFoot<R>& f = fq[fq_n + __popc(mm & lt_mask)];
-          f.x = nr.x;
-          f.y = nr.y;
-          f.nid = id;
-        }
-        fq_n += __popc(mm);
-        next += 32;
-        __syncwarp();
-        continue;
-      }
-      const int take_f = fq_n < 32 ? fq_n : 32;
-      bool hit = false;
-      Ray<R> nr;
-      int64_t id = 0;
-      if (lane < take_f) {
-        const QFoot<R>& f = fq[fq_n - take_f + lane];
-        id = f.nid;
-        nr.x = f.x;
-        nr.y = f.y;
-        nr.z = -Bm.z0;
-        nr.w = R(1);
-      }
-      fq_n -= take_f;
-      __syncwarp();
-      if (lane < take_f) {
-        const NeutronRng rng(A.keys, id);
-        R aux;
-        beam_divergence(Bm, rng, &nr, &aux);
-        Seg<R> seg[2 * NS];
-        const bool meets = assembly_segs<R, NS>(S, nr, seg) > 0;
-        const bool ok = (meets || !Bm.energy_positive) ? beam_energy(Bm, rng, aux, &nr) : true;
-        if (ok) {
-          if (meets)
-            hit = true;
-          else if (!(nr.w < S.min_prob))
-            T.bs.add(nr.w);  // order-0 packet, no material ahead
-        }
-      }
-      const unsigned hm = __ballot_sync(kFull, hit);
-      if (hit) {
-        QNeutron<R>& q = hq[hq_n + __popc(hm & lt_mask)];
-        q.x = nr.x;
-        q.y = nr.y;
-        q.z = nr.z;
-        q.dx = nr.dx;
-        q.dy = nr.dy;
-        q.dz = nr.dz;
-        q.speed = nr.speed;
-        q.t = nr.t;
-        q.nid = id;
-      }
-      hq_n += __popc(hm);
-      __syncwarp();
-    }
-    const int take = min(n_idle, hq_n);
+    n_beam += source_stage<R, NS, false>(A, job, n_idle, next, hi, src, q);
+    const int take = min(n_idle, q.hq_n);
     if (!busy) {
       const int r = __popc(idle & lt_mask);
       if (r < take) {
-        const QNeutron<R>& q = hq[hq_n - take + r];
-        cur.n.x = q.x;
-        cur.n.y = q.y;
-        cur.n.z = q.z;
-        cur.n.dx = q.dx;
-        cur.n.dy = q.dy;
-        cur.n.dz = q.dz;
-        cur.n.speed = q.speed;
-        cur.n.t = q.t;
-        cur.n.w = R(1);
+        nid = take_neutron<R>(job, q.hq[q.hq_n - take + r], &cur.n);
         cur.m = 0;
         cur.node = 1;
         cur.s0 = R(0);
-        nid = q.nid;
         sp = 0;
         jp = -1;
         have = true;
         busy = true;
       }
     }
-    hq_n -= take;
+    q.hq_n -= take;
     __syncwarp();
     // no lane has a tree only once the source queues are empty and the range is done
     if (!__any_sync(kFull, busy) && dq_n == 0) break;
@@ -475,7 +395,7 @@ __global__ void __launch_bounds__(kPaperThreads) paper_kernel(const __grid_const
     dq_n += __popc(em);
     __syncwarp();
     // detector stage: full batches of 32 packets, and the remainder at the end
-    const bool last = !__any_sync(kFull, busy) && hq_n == 0 && fq_n == 0 && next >= hi;
+    const bool last = !__any_sync(kFull, busy) && q.hq_n == 0 && q.fq_n == 0 && next >= hi;
     while (dq_n >= 32 || (last && dq_n > 0)) {
       const int take_d = dq_n < 32 ? dq_n : 32;
       PaperPk<R> p;
@@ -500,7 +420,7 @@ __global__ void __launch_bounds__(kPaperThreads) paper_kernel(const __grid_const
     const uint32_t n_miss = warp_sum(T.cnt.nmiss), n_hit = warp_sum(T.cnt.nhit);
     const uint32_t n_emit = warp_sum(T.cnt.nemit);
     if (lane == 0) {
-      atomicAdd(A.tallies + MCV_T_BEAMSTOP, v_bs);
+      atomicAdd(A.tallies + MCV_T_BEAMSTOP, v_bs + (double)n_beam);
       atomicAdd(A.tallies + MCV_T_WDET, v_det);
       atomicAdd(A.tallies + MCV_T_WOVER, v_over);
       atomicAdd(A.tallies + MCV_T_NDET, (double)n_det);

@@ -29,9 +29,10 @@ struct BeamP {
   // every energy draw is positive: rel z > -1 for every Box-Muller z the uniforms can give
   // (|z| <= sqrt(-2 ln 2^-54) = 8.65 for uniforms >= 2^-54), checked as rel * 8.7 < 1
   int energy_positive;
-  // footprints with |x| > x_safe or |y| > y_safe miss the sample for every divergence the
-  // uniforms can give (+inf: no such shortcut); set from the sample's bounding cylinder
-  R x_safe, y_safe;
+  // footprints that miss the sample for every divergence the uniforms can give: the leading
+  // 32 bits of the x (y) uniform below fx_lo (fy_lo) or above fx_hi (fy_hi); 0 and 2^32 - 1
+  // where there is no such shortcut.  Set from the sample's bounding cylinder.
+  uint32_t fx_lo, fx_hi, fy_lo, fy_hi;
 };
 
 template <typename R>

@@ -83,6 +83,13 @@ MCV_S64 uint64_t mul_hi32(uint64_t a, uint32_t y) {
   return (uint64_t)(uint32_t)(a >> 32) * y + (((uint64_t)(uint32_t)a * y) >> 32);
 }
 
+// operands outside the ranges of the functions below, out of their way
+MCV_S64_CALL double native_div(double a, double b) { return a / b; }
+MCV_S64_CALL double native_sqrt(double x) { return ::sqrt(x); }
+MCV_S64_CALL double native_exp(double x) { return ::exp(x); }
+MCV_S64_CALL double native_log(double x) { return ::log(x); }
+MCV_S64_CALL double native_tan(double x) { return ::tan(x); }
+
 // The reciprocal of a divisor, to be used for one or more quotients.
 struct Recip {
   double b;       // the divisor
@@ -117,7 +124,7 @@ MCV_S64 double div(double a, const Recip& r) {
   const int e0 = ea - eb + 1023;
   // both normal and the quotient normal whatever its rounding
   if (!((unsigned)(ea - 1) < 2046u && (unsigned)(eb - 1) < 2046u && (unsigned)(e0 - 2) < 2043u))
-    return a / r.b;
+    return native_div(a, r.b);
   const uint64_t ma = (A & 0xfffffffffffffull) | 0x10000000000000ull;
   const uint64_t mb = (B & 0xfffffffffffffull) | 0x10000000000000ull;
   uint64_t q = mul_hi64(ma << 11, r.y);  // a/b in (0.5, 2) in units of 2^-63, a few units off
@@ -137,12 +144,15 @@ MCV_S64 double div(double a, const Recip& r) {
 }
 
 MCV_S64_CALL double div(double a, double b) { return div(a, recip(b)); }
+// the same in two calls: the reciprocal's fixed-point significand, then the quotients
+MCV_S64_CALL uint64_t recip_of(double b) { return recip(b).y; }
+MCV_S64_CALL double div_by(double a, double b, uint64_t y) { return div(a, Recip{b, y}); }
 
 // sqrt(x), rounded to nearest even
 MCV_S64_CALL double sqrt(double x) {
   const uint64_t X = bits(x);
   const int e = (int)(X >> 52);  // with the sign bit: negative numbers leave the range below
-  if (!((unsigned)(e - 1) < 2046u)) return ::sqrt(x);
+  if (!((unsigned)(e - 1) < 2046u)) return native_sqrt(x);
   const uint64_t mx = (X & 0xfffffffffffffull) | 0x10000000000000ull;
   const int odd = (e & 1) ? 0 : 1;             // unbiased exponent odd: significand in [2, 4)
   const uint64_t v = mx << (10 + odd);         // in [1, 4), units of 2^-62
@@ -231,7 +241,7 @@ MCV_S64_CALL Pair sincos2pi(double u) {
 // exp(x); -700 <= x <= 0 in fixed point, other arguments by the library
 MCV_S64_CALL double exp(double x) {
   const uint64_t A = bits(x);
-  if (!(A >= 0x8000000000000000ull && A <= 0xc085e00000000000ull)) return ::exp(x);
+  if (!(A >= 0x8000000000000000ull && A <= 0xc085e00000000000ull)) return native_exp(x);
   const int e = ((int)(A >> 52) & 0x7ff) - 1023;
   if (e < -54) return 1.0;
   const uint64_t mx = (A & 0xfffffffffffffull) | 0x10000000000000ull;
@@ -270,7 +280,7 @@ MCV_S64_CALL double exp(double x) {
 MCV_S64_CALL double log(double x) {
   const uint64_t A = bits(x);
   const int e = (int)(A >> 52) - 1023;
-  if (!((unsigned)(e + 62) < 124u)) return ::log(x);
+  if (!((unsigned)(e + 62) < 124u)) return native_log(x);
   const uint64_t mx = (A & 0xfffffffffffffull) | 0x10000000000000ull;
   // x = 2^k m with m in (0.707, 1.414): significands above sqrt(2) are halved
   const bool half = mx > 0x16a09e667f3bcdull;
@@ -315,7 +325,7 @@ MCV_S64_CALL double log(double x) {
 MCV_S64_CALL double tan(double x) {
   const uint64_t A = bits(x);
   const int e = ((int)(A >> 52) & 0x7ff) - 1023;
-  if (!((unsigned)(e + 60) < 56u)) return ::tan(x);
+  if (!((unsigned)(e + 60) < 56u)) return native_tan(x);
   const uint64_t v = ((A & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
   const uint64_t f = v >> (-e - 1);                         // |x| < 2^-4, units of 2^-64
   const uint64_t w = mul_hi64(f, f);
@@ -332,6 +342,43 @@ MCV_S64_CALL double tan(double x) {
   const uint64_t q = (v >> 1) + (mul_hi64(v, mul_hi64(t, w)) >> 1);  // in [2^62, 2^63.01)
   const int l = leading_zeros(q);
   return pack(A & 0x8000000000000000ull, q << l, e + 1 - l);
+}
+
+// ---- tests and conversions (an FP64 comparison or conversion costs what an FP64 addition does,
+// 64 cycles; these are 2 to 15 integer instructions.  General comparisons, with NaN and signed
+// zeros some 20 instructions each, were slower inlined than the FP64 pipe's: code size) ------
+MCV_S64 bool is_zero(double x) { return (bits(x) << 1) == 0; }
+// a < b for a, b >= 0 that are not NaN
+MCV_S64 bool lt_nonneg(double a, double b) { return (int64_t)bits(a) < (int64_t)bits(b); }
+MCV_S64 bool positive(double x) {
+  const int64_t b = (int64_t)bits(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+// floor(x) where 0 <= x < n (n < 2^31), else -1
+MCV_S64 int index_below(double x, int n) {
+  const uint64_t b = bits(x);
+  const int e = (int)(b >> 52);
+  if (e < 1023 || b == 0x8000000000000000ull) return n > 0 ? 0 : -1;
+  if (e >= 1023 + 31) return -1;  // too large, negative (the sign bit) or NaN
+  const uint32_t m = (uint32_t)(((b & 0xfffffffffffffull) | 0x10000000000000ull) >> (1075 - e));
+  return m < (uint32_t)n ? (int)m : -1;
+}
+// floor(x) clamped to 0 .. n - 1 (NaN: 0)
+MCV_S64 int index_clamped(double x, int n) {
+  const uint64_t b = bits(x);
+  const int e = (int)(b >> 52);
+  if (e < 1023 || e > 2047 || b > 0x7ff0000000000000ull) return 0;
+  if (e >= 1023 + 31) return n - 1;
+  const uint32_t m = (uint32_t)(((b & 0xfffffffffffffull) | 0x10000000000000ull) >> (1075 - e));
+  return m < (uint32_t)n ? (int)m : n - 1;
+}
+// (2 k + 1) 2^-54 for the 53 bits k = hi 2^21 + (lo >> 11), rounded to nearest even
+MCV_S64 double uniform53(uint32_t hi, uint32_t lo) {
+  const uint64_t m = ((uint64_t)hi << 22) | (lo >> 10) | 1u;
+  const int lz = leading_zeros(m);  // 10 or more: only 54-bit values round, and those are ties
+  const uint64_t v = m << lz;
+  const uint64_t q = v >> 11;
+  return from_bits(((uint64_t)(unsigned)(1031 - lz) << 52) + q + ((v >> 10) & q & 1u));
 }
 
 }  // namespace soft64

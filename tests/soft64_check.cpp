@@ -80,7 +80,29 @@ int main(int argc, char** argv) {
       e_sc = std::fmax(e_sc, (double)std::fabs((long double)v[k] - w[k]) - half);
     }
   }
-  std::printf("{\"div_bad\": %ld, \"sqrt_bad\": %ld, \"log\": %.6g, \"exp\": %.6g, \"tan\": %.6g, "
-              "\"sincos\": %.6g, \"exp0\": %.17g, \"log1\": %.17g}\n", div_bad, sqrt_bad, e_log, e_exp,
+  // the integer tests and conversions
+  long conv_bad = 0;
+  for (long i = 0; i < n; ++i) {
+    double a = from_bits(r()), b = from_bits(r());
+    if (i % 3 == 1) a = std::ldexp((double)(r() >> 11), -50 + (int)(r() % 30)) * ((r() & 1) ? 1 : -1);
+    if (i % 3 == 2) a = special[r() % 11];
+    if (a != a) a = NAN;
+    conv_bad += positive(a) != (a > 0);
+    conv_bad += is_zero(a) != (a == 0);
+    const double c = std::fabs(a), e = std::fabs(b);
+    if (c == c && e == e) conv_bad += lt_nonneg(c, e) != (c < e);
+    const int m = 1 + (int)(r() % 2000);
+    const double f = std::floor(a);
+    conv_bad += index_below(a, m) != ((f >= 0 && f < m) ? (int)f : -1);
+    conv_bad += index_clamped(a, m) != (!(f > 0) ? 0 : f >= m ? m - 1 : (int)f);
+    uint32_t h = (uint32_t)r(), l = (uint32_t)r();
+    if (i % 5 == 0) h >>= r() % 32;
+    if (i % 50 == 0) h = 0;
+    if (i % 7 == 0) h = ~0u - (uint32_t)(r() % 3);
+    const uint64_t k = ((uint64_t)h << 21) | (l >> 11);
+    conv_bad += uniform53(h, l) != std::fma((double)k, 0x1p-53, 0x1p-54);
+  }
+  std::printf("{\"conv_bad\": %ld, \"div_bad\": %ld, \"sqrt_bad\": %ld, \"log\": %.6g, \"exp\": %.6g, \"tan\": %.6g, "
+              "\"sincos\": %.6g, \"exp0\": %.17g, \"log1\": %.17g}\n", conv_bad, div_bad, sqrt_bad, e_log, e_exp,
               e_tan, e_sc, mcv::soft64::exp(0.0), mcv::soft64::log(1.0));
 }
