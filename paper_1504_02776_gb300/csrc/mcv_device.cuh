@@ -1121,6 +1121,54 @@ __device__ __forceinline__ BvkPoint<R> bvk_point(const SampleP<R>& S, R c, R s, 
   return P;
 }
 
+// FP64 root search.  An FP64 evaluation of g costs some 300 FP64 instructions (an eigen-solve and
+// six sines), 64 cycles each, and the 33 nodes and 50 bisection steps took 84 of them.  The sign
+// of g is that of omega_b against the energy transfer, i.e. how many eigenvalues of D lie below
+// lambda* = (Ei - Ef)^2 / (hbar^2 phi/M): the sign changes along the leading minors of
+// D - lambda* (Sturm), a few dozen FP32 operations.  bvk_sign evaluates them with a bound on
+// their FP32 errors and answers +1 or -1 only where all three are beyond it, else 0; FP64 then
+// decides the nodes and bisection steps left (5 to 10 per event), and a bracketed secant
+// iteration (regula falsi, Illinois variant) takes the place of the remaining steps.
+// FP64 crystal, 5e4 neutrons: 25.1 -> 6.1 ms.
+static __device__ __noinline__ double bvk_g64(const SampleP<double>& S, double c, double s, double Ei,
+                                             double ki, double dix, double diy, double diz,
+                                             double dfx, double dfy, double dfz, double Ef, int b,
+                                             int sg) {
+  return bvk_point<double>(S, c, s, Ei, ki, dix, diy, diz, dfx, dfy, dfz, Ef, b, sg).g;
+}
+
+struct BvkSign {
+  float ax, ay, az, bx, by, bz;  // half-cell phases: a - kf b
+  float ei, inv_hwu;
+  int b, sg;
+  __device__ __forceinline__ int operator()(double Ef) const {
+    const float ef = (float)Ef;
+    const float kf = (float)kKPerV * sqrtf(ef / (float)kMeVPerV2);
+    const float x = ax - kf * bx, y = ay - kf * by, z = az - kf * bz;
+    float sx, cx, sy, cy, sz, cz;
+    sincosf(x, &sx, &cx);
+    sincosf(y, &sy, &cy);
+    sincosf(z, &sz, &cz);
+    const float t = (float)sg * (ei - ef) * inv_hwu;
+    const float lam = t * t;
+    const float d0 = 4.0f - 2.0f * cx * (cy + cz) - lam, d1 = 4.0f - 2.0f * cy * (cx + cz) - lam,
+                d2 = 4.0f - 2.0f * cz * (cx + cy) - lam;
+    const float e01 = 2.0f * sx * sy, e02 = 2.0f * sx * sz, e12 = 2.0f * sy * sz;
+    const float m2 = d0 * d1 - e01 * e01;
+    const float m3 = d2 * m2 - e12 * (d0 * e12 - e01 * e02) + e02 * (e01 * e12 - d1 * e02);
+    // entries are within err: the phases' FP32 rounding and that of lambda* (an energy transfer
+    // below 0.1 % of Ei + Ef is left to FP64); minors of entries up to S within 4 S err, 12 S^2 err
+    const float err = 2e-6f * (10.0f + fabsf(x) + fabsf(y) + fabsf(z)) + 8e-7f * t * (ei + ef) * inv_hwu;
+    const float S = 8.0f + lam;
+    if (!(t > 1e-3f * (ei + ef) * inv_hwu && fabsf(d0) > err && fabsf(m2) > 4.0f * S * err &&
+          fabsf(m3) > 12.0f * S * S * err))
+      return 0;
+    const int below = (d0 < 0.0f) + ((m2 < 0.0f) != (d0 < 0.0f)) + ((m3 < 0.0f) != (m2 < 0.0f));
+    const bool lower = below > b;  // omega_b below the energy transfer
+    return lower == (sg > 0) ? 1 : -1;
+  }
+};
+
 template <typename R, class Rng>
 __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
                                            const Rng& rng, int o, Ray<R>* n,
@@ -1146,10 +1194,40 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
   const R step = (hi - lo) / (R)kM;
   // signs of g on the grid, one bit per node
   uint64_t pos = 0;
-  for (int k = 0; k <= kM; ++k) {
-    const BvkPoint<R> P = bvk_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz,
-                                       lo + (R)k * step, b, sg);
-    if (M::positive(P.g)) pos |= (uint64_t)1 << k;
+  BvkSign quick;
+  if constexpr (sizeof(R) == 8) {
+    R qx, qy, qz;
+    to_crystal<R>(crot, srot, n->dx * ki, n->dy * ki, n->dz * ki, &qx, &qy, &qz);
+    quick.ax = (float)(S.bvk_ah * qx);
+    quick.ay = (float)(S.bvk_ah * qy);
+    quick.az = (float)(S.bvk_ah * qz);
+    to_crystal<R>(crot, srot, dfx, dfy, dfz, &qx, &qy, &qz);
+    quick.bx = (float)(S.bvk_ah * qx);
+    quick.by = (float)(S.bvk_ah * qy);
+    quick.bz = (float)(S.bvk_ah * qz);
+    quick.ei = (float)Ei;
+    quick.inv_hwu = (float)soft64::div(1.0, S.bvk_hwu);
+    quick.b = b;
+    quick.sg = sg;
+    uint64_t open = 0;
+    for (int k = 0; k <= kM; ++k) {
+      const int sign = quick(lo + (R)k * step);
+      if (sign > 0) pos |= (uint64_t)1 << k;
+      if (sign == 0) open |= (uint64_t)1 << k;
+    }
+    while (open) {  // each lane its own undecided nodes
+      const int k = __ffsll((long long)open) - 1;
+      open &= open - 1;
+      if (M::positive(bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz,
+                              lo + (R)k * step, b, sg)))
+        pos |= (uint64_t)1 << k;
+    }
+  } else {
+    for (int k = 0; k <= kM; ++k) {
+      const BvkPoint<R> P = bvk_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz,
+                                         lo + (R)k * step, b, sg);
+      if (M::positive(P.g)) pos |= (uint64_t)1 << k;
+    }
   }
   const uint64_t change = (pos ^ (pos >> 1)) & ((((uint64_t)1) << kM) - 1);
   const int nroots = __popcll(change);
@@ -1161,15 +1239,54 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
   const int kb = __ffsll((long long)ch) - 1;
   R ea = lo + (R)kb * step, eb = lo + (R)(kb + 1) * step;
   const bool ga_pos = (pos >> kb) & 1;
-  const int iters = sizeof(R) == 8 ? 50 : 24;
-  for (int it = 0; it < iters; ++it) {
-    const R mid = R(0.5) * (ea + eb);
-    const BvkPoint<R> P = bvk_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz,
-                                       mid, b, sg);
-    if (M::positive(P.g) == ga_pos)
-      ea = mid;
-    else
-      eb = mid;
+  if constexpr (sizeof(R) == 8) {
+    // bisection while the FP32 sign is certain, then the secant iteration on the FP64 bracket
+    for (int it = 0; it < 50; ++it) {
+      const R mid = R(0.5) * (ea + eb);
+      const int sign = quick(mid);
+      if (sign == 0) break;
+      if ((sign > 0) == ga_pos)
+        ea = mid;
+      else
+        eb = mid;
+    }
+    R ga = bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz, ea, b, sg);
+    R gb = bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz, eb, b, sg);
+    int side = 0;
+    for (int it = 0; it < 60; ++it) {
+      const R w = eb - ea;
+      if (!(w > 2.3e-16 * eb)) break;  // neighbouring doubles
+      // (every fourth step halves the bracket, so that it closes whatever the function)
+      R mid = (it & 3) == 3 ? R(0.5) * (ea + eb) : ea + w * M::div(ga, ga - gb);
+      if (!(mid > ea && mid < eb)) mid = R(0.5) * (ea + eb);
+      if (!(mid > ea && mid < eb)) break;
+      const R g = bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz, mid, b, sg);
+      if (!(M::fabs(g) > 2e-16 * (Ei + mid))) {  // the rounding of Ei - Ef
+        ea = eb = mid;
+        break;
+      }
+      if (M::positive(g) == ga_pos) {
+        ea = mid;
+        ga = g;
+        if (side == 1) gb *= R(0.5);
+        side = 1;
+      } else {
+        eb = mid;
+        gb = g;
+        if (side == -1) ga *= R(0.5);
+        side = -1;
+      }
+    }
+  } else {
+    for (int it = 0; it < 24; ++it) {
+      const R mid = R(0.5) * (ea + eb);
+      const BvkPoint<R> P = bvk_point<R>(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz,
+                                         mid, b, sg);
+      if (M::positive(P.g) == ga_pos)
+        ea = mid;
+      else
+        eb = mid;
+    }
   }
   const R Ef = R(0.5) * (ea + eb);
   if (!(Ef > R(0))) return false;
