@@ -212,10 +212,16 @@ struct SourceQueues {
 // sample stage, the rest add to the beam stop.  (Misses need no energy: the footprint bounds
 // are set only when every energy draw is positive.)  DROP: neutrons lighter than min_prob are
 // dropped here.  Returns the neutrons of weight 1 that miss the sample, the same in every lane.
-template <typename R, int NS, bool DROP, class Job, class Src>
+// miss(): called by each lane whose neutron misses, where Miss::kPerLane (the FP32 waves add them
+// to the lane's compensated sum one by one, whose rounding the tallies keep).
+struct CountMisses {
+  static constexpr bool kPerLane = false;
+  __device__ __forceinline__ void operator()() const {}
+};
+template <typename R, int NS, bool DROP, class Job, class Src, class Miss = CountMisses>
 __device__ __forceinline__ uint32_t source_stage(const TraceArgs& A, const Job& job, int need,
                                                  int64_t& next, int64_t& hi, Src& src,
-                                                 SourceQueues<R>& q) {
+                                                 SourceQueues<R>& q, const Miss& on_miss = Miss()) {
   const SampleP<R>& S = job.S();
   const unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -229,6 +235,7 @@ __device__ __forceinline__ uint32_t source_stage(const TraceArgs& A, const Job& 
       if (i < hi) {
         w = job.rng(job.first_id() + i).words(-1, 1);
         maybe = !footprint_misses<R>(job.B(), w);
+        if (Miss::kPerLane && !maybe && !(R(1) < S.min_prob)) on_miss();
       }
       const unsigned mm = __ballot_sync(kFull, maybe);
       if (maybe)
@@ -262,6 +269,7 @@ __device__ __forceinline__ uint32_t source_stage(const TraceArgs& A, const Job& 
                                                           : true;
       hit = ok && meets;
       miss = ok && !meets;
+      if (Miss::kPerLane && miss && !(R(1) < S.min_prob)) on_miss();
       if (DROP) hit = hit && !(nr.w < S.min_prob) && !(A.stop_on_zero && nr.w == R(0));
     }
     const unsigned hm = __ballot_sync(kFull, hit);
@@ -282,7 +290,7 @@ __device__ __forceinline__ uint32_t source_stage(const TraceArgs& A, const Job& 
     __syncwarp();
   }
   // a neutron of weight 1 counts at the beam stop unless it is lighter than min_prob
-  return R(1) < S.min_prob ? 0u : missed;
+  return Miss::kPerLane || R(1) < S.min_prob ? 0u : missed;
 }
 
 // a queued neutron as a packet of order 0; returns its id
@@ -514,6 +522,14 @@ struct WaveSink {
   }
 };
 
+// the FP32 waves' neutrons of weight 1 that miss the sample, into the lane's beam-stop sum
+template <typename R, class P>
+struct LaneMisses {
+  static constexpr bool kPerLane = sizeof(R) == 4;
+  P& pol;
+  __device__ __forceinline__ void operator()() const { pol.sums().bs.add(R(1)); }
+};
+
 // The waves of one warp over neutron ids first_id + [lo, hi) of one simulation, and over
 // every further range `src` hands out for it.  Returns with both queues empty.
 // FORM: see detect().
@@ -543,7 +559,8 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
     const unsigned idle = __ballot_sync(kFull, !L.active);
     const int n_idle = __popc(idle);
     // ---- source stage
-    const uint32_t n_beam = source_stage<R, NS, true>(A, job, n_idle, next, hi, src, q);
+    const LaneMisses<R, P> on_miss{pol};
+    const uint32_t n_beam = source_stage<R, NS, true>(A, job, n_idle, next, hi, src, q, on_miss);
     const int take = min(n_idle, q.hq_n);
     if (!L.active) {
       const int r = __popc(idle & lt_mask);
