@@ -25,3 +25,7 @@ def errors(tmp_path_factory):
 
 def test_sin_and_cos_are_relatively_accurate(errors):
     assert errors["sincos"] <= 0.52, errors
+
+
+def test_exp_is_accurate_down_to_its_smallest_values(errors):
+    assert errors["exp"] <= 0.52, errors
