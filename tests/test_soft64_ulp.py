@@ -29,3 +29,7 @@ def test_sin_and_cos_are_relatively_accurate(errors):
 
 def test_exp_is_accurate_down_to_its_smallest_values(errors):
     assert errors["exp"] <= 0.52, errors
+
+
+def test_log_is_accurate_next_to_one(errors):
+    assert errors["log"] <= 0.52, errors
