@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "mcv_bvk_sign.cuh"
 #include "mcv_params.h"
 #include "mcv_soft64.cuh"
 
@@ -1121,53 +1122,13 @@ __device__ __forceinline__ BvkPoint<R> bvk_point(const SampleP<R>& S, R c, R s, 
   return P;
 }
 
-// FP64 root search.  An FP64 evaluation of g costs some 300 FP64 instructions (an eigen-solve and
-// six sines), 64 cycles each, and the 33 nodes and 50 bisection steps took 84 of them.  The sign
-// of g is that of omega_b against the energy transfer, i.e. how many eigenvalues of D lie below
-// lambda* = (Ei - Ef)^2 / (hbar^2 phi/M): the sign changes along the leading minors of
-// D - lambda* (Sturm), a few dozen FP32 operations.  bvk_sign evaluates them with a bound on
-// their FP32 errors and answers +1 or -1 only where all three are beyond it, else 0; FP64 then
-// decides the nodes and bisection steps left (5 to 10 per event), and a bracketed secant
-// iteration (regula falsi, Illinois variant) takes the place of the remaining steps.
-// FP64 crystal, 5e4 neutrons: 25.1 -> 6.1 ms.
+// one FP64 evaluation of g, compiled once per kernel
 static __device__ __noinline__ double bvk_g64(const SampleP<double>& S, double c, double s, double Ei,
                                              double ki, double dix, double diy, double diz,
                                              double dfx, double dfy, double dfz, double Ef, int b,
                                              int sg) {
   return bvk_point<double>(S, c, s, Ei, ki, dix, diy, diz, dfx, dfy, dfz, Ef, b, sg).g;
 }
-
-struct BvkSign {
-  float ax, ay, az, bx, by, bz;  // half-cell phases: a - kf b
-  float ei, inv_hwu;
-  int b, sg;
-  __device__ __forceinline__ int operator()(double Ef) const {
-    const float ef = (float)Ef;
-    const float kf = (float)kKPerV * sqrtf(ef / (float)kMeVPerV2);
-    const float x = ax - kf * bx, y = ay - kf * by, z = az - kf * bz;
-    float sx, cx, sy, cy, sz, cz;
-    sincosf(x, &sx, &cx);
-    sincosf(y, &sy, &cy);
-    sincosf(z, &sz, &cz);
-    const float t = (float)sg * (ei - ef) * inv_hwu;
-    const float lam = t * t;
-    const float d0 = 4.0f - 2.0f * cx * (cy + cz) - lam, d1 = 4.0f - 2.0f * cy * (cx + cz) - lam,
-                d2 = 4.0f - 2.0f * cz * (cx + cy) - lam;
-    const float e01 = 2.0f * sx * sy, e02 = 2.0f * sx * sz, e12 = 2.0f * sy * sz;
-    const float m2 = d0 * d1 - e01 * e01;
-    const float m3 = d2 * m2 - e12 * (d0 * e12 - e01 * e02) + e02 * (e01 * e12 - d1 * e02);
-    // entries are within err: the phases' FP32 rounding and that of lambda* (an energy transfer
-    // below 0.1 % of Ei + Ef is left to FP64); minors of entries up to S within 4 S err, 12 S^2 err
-    const float err = 2e-6f * (10.0f + fabsf(x) + fabsf(y) + fabsf(z)) + 8e-7f * t * (ei + ef) * inv_hwu;
-    const float S = 8.0f + lam;
-    if (!(t > 1e-3f * (ei + ef) * inv_hwu && fabsf(d0) > err && fabsf(m2) > 4.0f * S * err &&
-          fabsf(m3) > 12.0f * S * S * err))
-      return 0;
-    const int below = (d0 < 0.0f) + ((m2 < 0.0f) != (d0 < 0.0f)) + ((m3 < 0.0f) != (m2 < 0.0f));
-    const bool lower = below > b;  // omega_b below the energy transfer
-    return lower == (sg > 0) ? 1 : -1;
-  }
-};
 
 template <typename R, class Rng>
 __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
@@ -1196,15 +1157,11 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
   uint64_t pos = 0;
   BvkSign quick;
   if constexpr (sizeof(R) == 8) {
-    R qx, qy, qz;
+    R qx, qy, qz, rx, ry, rz;
     to_crystal<R>(crot, srot, n->dx * ki, n->dy * ki, n->dz * ki, &qx, &qy, &qz);
-    quick.ax = (float)(S.bvk_ah * qx);
-    quick.ay = (float)(S.bvk_ah * qy);
-    quick.az = (float)(S.bvk_ah * qz);
-    to_crystal<R>(crot, srot, dfx, dfy, dfz, &qx, &qy, &qz);
-    quick.bx = (float)(S.bvk_ah * qx);
-    quick.by = (float)(S.bvk_ah * qy);
-    quick.bz = (float)(S.bvk_ah * qz);
+    to_crystal<R>(crot, srot, dfx, dfy, dfz, &rx, &ry, &rz);
+    quick.set_phases((float)(S.bvk_ah * qx), (float)(S.bvk_ah * qy), (float)(S.bvk_ah * qz),
+                     (float)(S.bvk_ah * rx), (float)(S.bvk_ah * ry), (float)(S.bvk_ah * rz));
     quick.ei = (float)Ei;
     quick.inv_hwu = (float)soft64::div(1.0, S.bvk_hwu);
     quick.b = b;

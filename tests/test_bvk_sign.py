@@ -1,0 +1,46 @@
+"""The FP32 signs of the FP64 single-crystal root search (csrc/mcv_bvk_sign.cuh).  On the CPU, as
+plain C++: the bound on the FP32 errors holds (every ratio at most 1, the bar the bound itself
+states) and no sign it calls certain is wrong, over cells of 2 to 60 A, stiffnesses, masses,
+energies and near-forward directions.  On the GPU: packets of stiff crystals with large cells
+against the oracle, with the FP64 per-packet bars of the parity tests."""
+import dataclasses
+import json
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import mcv_inputs as mi
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1504_02776_gb300", "csrc")
+
+
+def test_error_bound_holds_over_cells_and_energies(tmp_path):
+    exe = str(tmp_path / "bvk_sign_check")
+    subprocess.run(["g++", "-O2", "-std=gnu++17", "-ffp-contract=off", "-I" + CSRC, "-x", "c++",
+                    os.path.join(HERE, "bvk_sign_check.cpp"), "-o", exe], check=True)
+    got = json.loads(subprocess.run([exe, "2000000"], check=True, capture_output=True,
+                                    text=True).stdout)
+    assert got["wrong"] == 0, got
+    assert got["entry"] <= 1.0 and got["m2"] <= 1.0 and got["m3"] <= 1.0, got
+    assert got["open"] < 0.3, got
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("a,phi,mass,ei", [(12.0, 100.0, 12.0, 500.0), (30.0, 10.0, 27.0, 120.0)])
+def test_fp64_packets_of_large_cells_match_oracle(a, phi, mass, ei):
+    import oracle
+    from paper_1504_02776_gb300 import binding as B
+    import gpu_helpers as H
+    ctx = H.ctx()
+    wl = mi.config3(rot_deg=20.0, n=1500)
+    wl = wl.replace(beam=mi.powder_beam(ei=ei),
+                    bvk=dataclasses.replace(wl.bvk, a_A=a, phi_Nm=phi, mass_u=mass))
+    pk, g = H.packets(ctx, wl, B.FP64)
+    op = oracle.trace(wl, packets=True)["packets"]
+    dev, bad = H.check_fp64_packets(g, op)
+    assert not any(bad.values()), (bad, {f: float(d.max()) for f, d in dev.items()})
+    assert np.count_nonzero(op["order"] >= 1) > 100
+    ctx.close()
