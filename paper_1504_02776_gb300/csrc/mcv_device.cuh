@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "mcv_bracket.cuh"
 #include "mcv_bvk_sign.cuh"
 #include "mcv_params.h"
 #include "mcv_soft64.cuh"
@@ -1197,43 +1198,9 @@ __device__ __forceinline__ bool kernel_bvk(const SampleP<R>& S, R crot, R srot,
   R ea = lo + (R)kb * step, eb = lo + (R)(kb + 1) * step;
   const bool ga_pos = (pos >> kb) & 1;
   if constexpr (sizeof(R) == 8) {
-    // bisection while the FP32 sign is certain, then the secant iteration on the FP64 bracket
-    for (int it = 0; it < 50; ++it) {
-      const R mid = R(0.5) * (ea + eb);
-      const int sign = quick(mid);
-      if (sign == 0) break;
-      if ((sign > 0) == ga_pos)
-        ea = mid;
-      else
-        eb = mid;
-    }
-    R ga = bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz, ea, b, sg);
-    R gb = bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz, eb, b, sg);
-    int side = 0;
-    for (int it = 0; it < 60; ++it) {
-      const R w = eb - ea;
-      if (!(w > 2.3e-16 * eb)) break;  // neighbouring doubles
-      // (every fourth step halves the bracket, so that it closes whatever the function)
-      R mid = (it & 3) == 3 ? R(0.5) * (ea + eb) : ea + w * M::div(ga, ga - gb);
-      if (!(mid > ea && mid < eb)) mid = R(0.5) * (ea + eb);
-      if (!(mid > ea && mid < eb)) break;
-      const R g = bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz, mid, b, sg);
-      if (!(M::fabs(g) > 2e-16 * (Ei + mid))) {  // the rounding of Ei - Ef
-        ea = eb = mid;
-        break;
-      }
-      if (M::positive(g) == ga_pos) {
-        ea = mid;
-        ga = g;
-        if (side == 1) gb *= R(0.5);
-        side = 1;
-      } else {
-        eb = mid;
-        gb = g;
-        if (side == -1) ga *= R(0.5);
-        side = -1;
-      }
-    }
+    ea = eb = bracket_root(ea, eb, ga_pos, Ei, quick, [&](R ef) {
+      return bvk_g64(S, crot, srot, Ei, ki, n->dx, n->dy, n->dz, dfx, dfy, dfz, ef, b, sg);
+    });
   } else {
     for (int it = 0; it < 24; ++it) {
       const R mid = R(0.5) * (ea + eb);
