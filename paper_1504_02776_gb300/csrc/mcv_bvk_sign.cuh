@@ -6,8 +6,10 @@
 // of D lie below lambda* = (Ei - Ef)^2 / (hbar^2 phi/M): the sign changes along the leading
 // minors of D - lambda* (Sturm), a few dozen FP32 operations.  BvkSign evaluates them with a
 // bound on their FP32 errors and answers +1 or -1 only where all three are beyond it, else 0:
-// FP64 decides the nodes and bisection steps left (5 to 10 per event), and a bracketed secant
-// iteration takes the place of the remaining steps.  FP64 crystal, 5e4 neutrons: 25.1 -> 6.1 ms.
+// FP64 decides those (bracket_root).  The bound follows the entries' and cofactors' values: it
+// leaves 0.01 % of the points open where the signs are not (and the node at Ef = Ei), against
+// 2.2 % with one from the largest values they can have.  FP64 crystal, 5e4 neutrons: 25.1 ms
+// with FP64 throughout, 5.3 ms, and 8.3 ms with the wider bound.
 //
 // The header also compiles as plain C++ (a CPU test checks the bound over cells, stiffnesses and
 // energies there).
@@ -30,12 +32,12 @@ MCV_BVK void bvk_sincos(float x, float* s, float* c) { sincosf(x, s, c); }
 void bvk_sincos(float x, float* s, float* c);  // the test's: with errors of its choice
 #endif
 
-// the entries of D - lambda* in units of phi/M (xx yy zz xy xz yz), the bound on their errors and
-// on their magnitude
+// the entries of D - lambda* in units of phi/M (xx yy zz xy xz yz), the second and third leading
+// minors (the first is d0), and the bounds on the errors of the entries and of the minors
 struct BvkMinors {
   float d0, d1, d2, e01, e02, e12;
-  float m2, m3;  // the second and third leading minors; the first is d0
-  float err, size;
+  float m2, m3;
+  float err, err2, err3;
 };
 
 struct BvkSign {
@@ -64,9 +66,11 @@ struct BvkSign {
   //   entries:  40 u = 2.4e-6 for sines, cosines and their products
   //   lambda*:  t carries 4 u (ei + ef) inv_hwu, so lambda* 9.1 u t (ei + ef) inv_hwu, and its
   //             subtraction one u of it: 6.1e-7 t (ei + ef) inv_hwu
-  // The minors of entries that are within err, and at most S = 8 + lambda*, are within
-  // (2 S + 4) err and (3 S^2 + 12 S + 36) err, and their own rounding within 3 u S^2 and
-  // 6 u S^3: together below 4 S err and 12 S^2 err, since S >= 8 and err > 8e-7 lambda* + 2e-5.
+  // The minors of entries that are within err: a minor moves by err times the sum of its
+  // cofactors' magnitudes (off-diagonal ones twice), plus 2 err^2 (second) and 2 err^2 times the
+  // sum of the entries' magnitudes (third: adj(E) is at most 2 err^2), plus its own rounding, at
+  // most 3 u and 5 u of the sum of its products' magnitudes; 1.1 for the rounding of the bounds
+  // and the terms err^3.
   MCV_BVK BvkMinors minors(float ef, float t) const {
     const float kf = (float)kKPerV * sqrtf(ef / (float)kMeVPerV2);
     float sx, cx, sy, cy, sz, cz;
@@ -81,11 +85,21 @@ struct BvkSign {
     m.e01 = 2.0f * sx * sy;
     m.e02 = 2.0f * sx * sz;
     m.e12 = 2.0f * sy * sz;
+    const float c00 = m.d1 * m.d2 - m.e12 * m.e12, c11 = m.d0 * m.d2 - m.e02 * m.e02;
+    const float c01 = m.e02 * m.e12 - m.e01 * m.d2, c02 = m.e01 * m.e12 - m.e02 * m.d1,
+                c12 = m.e01 * m.e02 - m.e12 * m.d0;
     m.m2 = m.d0 * m.d1 - m.e01 * m.e01;
-    m.m3 = m.d2 * m.m2 - m.e12 * (m.d0 * m.e12 - m.e01 * m.e02) +
-           m.e02 * (m.e01 * m.e12 - m.d1 * m.e02);
-    m.err = 2e-6f * (10.0f + pa + kf * pb) + 8e-7f * t * (ei + ef) * inv_hwu;
-    m.size = 8.0f + lam;
+    m.m3 = m.d2 * m.m2 + m.e12 * c12 + m.e02 * c02;
+    m.err = 2e-6f * (2.0f + pa + kf * pb) + 8e-7f * t * (ei + ef) * inv_hwu;
+    const float a0 = fabsf(m.d0), a1 = fabsf(m.d1), a2 = fabsf(m.d2);
+    const float b01 = fabsf(m.e01), b02 = fabsf(m.e02), b12 = fabsf(m.e12);
+    const float p2 = a0 * a1 + b01 * b01;
+    const float p3 = a2 * p2 + b12 * (b12 * a0 + b01 * b02) + b02 * (b01 * b12 + b02 * a1);
+    m.err2 = 1.1f * (m.err * (a0 + a1 + 2.0f * (b01 + m.err)) + 1.8e-7f * p2);
+    m.err3 = 1.1f * (m.err * (fabsf(c00) + fabsf(c11) + fabsf(m.m2) +
+                              2.0f * (fabsf(c01) + fabsf(c02) + fabsf(c12)) +
+                              2.0f * m.err * (a0 + a1 + a2 + 2.0f * (b01 + b02 + b12))) +
+                     3e-7f * p3);
     return m;
   }
 
@@ -95,8 +109,8 @@ struct BvkSign {
     const float ef = (float)Ef;
     const float t = (float)sg * (ei - ef) * inv_hwu;
     const BvkMinors m = minors(ef, t);
-    if (!(t > 1e-3f * (ei + ef) * inv_hwu && fabsf(m.d0) > m.err &&
-          fabsf(m.m2) > 4.0f * m.size * m.err && fabsf(m.m3) > 12.0f * m.size * m.size * m.err))
+    if (!(t > 1e-3f * (ei + ef) * inv_hwu && fabsf(m.d0) > m.err && fabsf(m.m2) > m.err2 &&
+          fabsf(m.m3) > m.err3))
       return 0;
     const int below = (m.d0 < 0.0f) + ((m.m2 < 0.0f) != (m.d0 < 0.0f)) +
                       ((m.m3 < 0.0f) != (m.m2 < 0.0f));

@@ -1,6 +1,6 @@
 // Checks csrc/mcv_bvk_sign.cuh as plain C++ against the same matrix in double: the entries of
-// D - lambda* against the bound `err`, the minors against their multiples of it, and every sign
-// that is not left undecided.  Cells, stiffnesses, masses, energies, directions (near forward
+// D - lambda* against the bound `err`, the minors against theirs, and every sign that is not left
+// undecided.  Cells, stiffnesses, masses, energies, directions (near forward
 // among them) and modes are drawn; sine and cosine are off by up to two units in the last place.
 // Prints one JSON object: the largest error over its bound, the wrong signs, and the share of
 // undecided ones.
@@ -84,8 +84,8 @@ int main(int argc, char** argv) {
     const mcv::BvkMinors m = q.minors(ef, tf);
     const double pairs[6][2] = {{m.d0, d0}, {m.d1, d1}, {m.d2, d2}, {m.e01, e01}, {m.e02, e02}, {m.e12, e12}};
     for (const auto& p : pairs) r_entry = std::fmax(r_entry, std::fabs(p[0] - p[1]) / m.err);
-    r_m2 = std::fmax(r_m2, std::fabs(m.m2 - m2) / (4.0 * m.size * m.err));
-    r_m3 = std::fmax(r_m3, std::fabs(m.m3 - m3) / (12.0 * m.size * m.size * m.err));
+    r_m2 = std::fmax(r_m2, std::fabs(m.m2 - m2) / m.err2);
+    r_m3 = std::fmax(r_m3, std::fabs(m.m3 - m3) / m.err3);
     if (got == 0) {
       ++open;
       continue;

@@ -25,7 +25,7 @@ def test_error_bound_holds_over_cells_and_energies(tmp_path):
                                     text=True).stdout)
     assert got["wrong"] == 0, got
     assert got["entry"] <= 1.0 and got["m2"] <= 1.0 and got["m3"] <= 1.0, got
-    assert got["open"] < 0.3, got
+    assert got["open"] < 0.1, got
 
 
 @pytest.mark.gpu
