@@ -557,6 +557,17 @@ int grid_for(mcv_ctx* ctx, int64_t items, int per_sm) {
   return (int)(g < 1 ? 1 : g);
 }
 
+// resident blocks per SM of the kernel that traces A
+int trace_blocks(mcv_ctx* ctx, const mcv::TraceArgs& A, int fp, int det) {
+  const int waves = mcv::uses_waves(A, det) ? 1 : 0;
+  int& occ = ctx->occ[fp][ns_index(A.Sd.ns)][det][A.Sd.wide ? 1 : 0][waves];
+  if (occ == 0) {
+    cudaError_t e = mcv::trace_blocks_per_sm(fp, A.Sd.ns, det, A.Sd.wide, waves, &occ);
+    if (e != cudaSuccess || occ < 1) occ = 1;
+  }
+  return occ;
+}
+
 PhiloxKeys philox_keys(uint32_t seed, uint32_t sim_id) {
   PhiloxKeys K;
   uint32_t k0 = seed, k1 = sim_id;
@@ -822,12 +833,7 @@ mcv_status mcv_trace_sample(mcv_ctx* ctx, const mcv_sample* sample, const mcv_be
     if (e != cudaSuccess) return cuda_fail(e, "paper kernel launch");
     return MCV_OK;
   }
-  int& occ = ctx->occ[fp][ns_index(A.Sd.ns)][detk][A.Sd.wide ? 1 : 0];
-  if (occ == 0) {
-    cudaError_t e = mcv::trace_blocks_per_sm(fp, A.Sd.ns, detk, A.Sd.wide, &occ);
-    if (e != cudaSuccess || occ < 1) occ = 1;
-  }
-  const int grid = grid_for(ctx, n, occ);
+  const int grid = grid_for(ctx, n, trace_blocks(ctx, A, fp, detk));
   cast_all(&A);
   cudaError_t e = mcv::launch_trace(A, fp, detk, grid, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "trace kernel launch");
@@ -982,12 +988,7 @@ mcv_status mcv_grad(mcv_ctx* ctx, const mcv_sample* sample, const mcv_beam_param
     A.hist = hist->counts;
     A.tallies = hist->tallies;
     A.stop_on_zero = 1;
-    int& occ = ctx->occ[fp][ns_index(A.Sd.ns)][A.Dd.kind][A.Sd.wide ? 1 : 0];
-    if (occ == 0) {
-      e = mcv::trace_blocks_per_sm(fp, A.Sd.ns, A.Dd.kind, A.Sd.wide, &occ);
-      if (e != cudaSuccess || occ < 1) occ = 1;
-    }
-    e = mcv::launch_trace(A, fp, A.Dd.kind, grid_for(ctx, n, occ), s);
+    e = mcv::launch_trace(A, fp, A.Dd.kind, grid_for(ctx, n, trace_blocks(ctx, A, fp, A.Dd.kind)), s);
     if (e != cudaSuccess) return cuda_fail(e, "trace kernel launch");
   }
   return loss_and_adjoint(ctx, A, fp, hist->counts, target, scale_c, g_work, loss, dsqe, dsig, s);

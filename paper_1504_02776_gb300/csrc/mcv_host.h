@@ -15,7 +15,8 @@ struct mcv_ctx {
   int device;
   int sm_count;
   int* d_err;          // device error flag (kernels set it; mcv_sync reads and clears it)
-  int occ[2][3][3][2]; // cached blocks per SM of the fused kernel: [fp][ns 1,2,4][det][bvk]
+  // cached blocks per SM of the trace kernels: [fp][ns 1,2,4][det][bvk][waves]
+  int occ[2][3][3][2][2];
   int occ_adj[2][3][3][2];  // the same for the adjoint kernel
   // batched launch chosen by mcv_batch_tune for a kind of batch: neutrons per work item and
   // blocks per SM (0: not tuned yet); [fp][ns 1,2,4][det][bvk][one sample for all]

@@ -777,12 +777,6 @@ __global__ void __launch_bounds__(WaveCfg<R>::threads, 1)
   }
 }
 
-// the fused forward runs as waves (dynamic shared memory for the warp queues) unless it
-// stores packets or reads a stored beam
-inline bool uses_waves(const TraceArgs& A, int det) {
-  return det != MCV_DET_NONE && A.pk_order == nullptr && A.in_x == nullptr;
-}
-
 template <typename R>
 __global__ void __launch_bounds__(kThreads) beam_kernel(const __grid_constant__ TraceArgs A) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < A.n;
@@ -1176,25 +1170,31 @@ cudaError_t launch_trace_t(const TraceArgs& A, int det, int grid, cudaStream_t s
   return launch_trace_ns<R, 4>(A, det, grid, s);
 }
 
-// the kernel the fused forward of this shape launches (waves when a detector is fused)
+// the kernel that launch_trace launches for this shape: the waves, or one neutron per lane (a
+// stored beam or packet slots)
 template <typename R, int NS, int KS>
-const void* trace_fn_nk(int det) {
-  if (det == MCV_DET_SURFACE) return (const void*)wave_kernel<R, NS, MCV_DET_SURFACE, KS, false>;
-  if (det == MCV_DET_TUBES) return (const void*)wave_kernel<R, NS, MCV_DET_TUBES, KS, false>;
+const void* trace_fn_nk(int det, bool waves) {
+  if (det == MCV_DET_SURFACE)
+    return waves ? (const void*)wave_kernel<R, NS, MCV_DET_SURFACE, KS, false>
+                 : (const void*)trace_kernel<R, NS, MCV_DET_SURFACE, KS>;
+  if (det == MCV_DET_TUBES)
+    return waves ? (const void*)wave_kernel<R, NS, MCV_DET_TUBES, KS, false>
+                 : (const void*)trace_kernel<R, NS, MCV_DET_TUBES, KS>;
   return (const void*)trace_kernel<R, NS, MCV_DET_NONE, KS>;
 }
 
 template <typename R, int NS>
-const void* trace_fn_ns(int det, bool bvk) {
-  return bvk ? trace_fn_nk<R, NS, kKernelsAll>(det) : trace_fn_nk<R, NS, kKernelsPowder>(det);
+const void* trace_fn_ns(int det, bool bvk, bool waves) {
+  return bvk ? trace_fn_nk<R, NS, kKernelsAll>(det, waves)
+             : trace_fn_nk<R, NS, kKernelsPowder>(det, waves);
 }
 
 template <typename R>
-cudaError_t blocks_per_sm_t(int ns, int det, int bvk, int* blocks) {
-  const void* fn = ns <= 1 ? trace_fn_ns<R, 1>(det, bvk) : (ns == 2 ? trace_fn_ns<R, 2>(det, bvk)
-                                                                    : trace_fn_ns<R, 4>(det, bvk));
-  if (det == MCV_DET_NONE)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kThreads, 0);
+cudaError_t blocks_per_sm_t(int ns, int det, int bvk, int waves, int* blocks) {
+  const void* fn = ns <= 1 ? trace_fn_ns<R, 1>(det, bvk, waves)
+                           : (ns == 2 ? trace_fn_ns<R, 2>(det, bvk, waves)
+                                      : trace_fn_ns<R, 4>(det, bvk, waves));
+  if (!waves) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kThreads, 0);
   cudaError_t e = allow_wave_smem<R>(fn, false);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
@@ -1335,8 +1335,8 @@ cudaError_t launch_paper_t(const TraceArgs& A, int det, int grid, cudaStream_t s
     return launch_trace_t<R>(A, det, grid, s);                                              \
   }                                                                                         \
   int wave_threads_##SUFFIX() { return WaveCfg<R>::threads; }                               \
-  cudaError_t blocks_per_sm_##SUFFIX(int ns, int det, int bvk, int* blocks) {               \
-    return blocks_per_sm_t<R>(ns, det, bvk, blocks);                                        \
+  cudaError_t blocks_per_sm_##SUFFIX(int ns, int det, int bvk, int waves, int* blocks) {    \
+    return blocks_per_sm_t<R>(ns, det, bvk, waves, blocks);                                 \
   }
 
 // the fused waves with an event list (mcv_fp32_ev.cu / mcv_fp64_ev.cu)

@@ -17,10 +17,17 @@ struct EventsArgs {
   int64_t* bin;
 };
 
+// the fused forward runs as waves (dynamic shared memory for the warp queues) unless it stores
+// packets or reads a stored beam
+inline bool uses_waves(const TraceArgs& A, int det) {
+  return det != MCV_DET_NONE && A.pk_order == nullptr && A.in_x == nullptr;
+}
+
 int trace_threads();
 // threads per block of the fused (waves) and batched kernels
 int wave_threads(int fp_mode);
-cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int* blocks);
+// resident blocks per SM of the kernel launch_trace launches; waves: uses_waves
+cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int waves, int* blocks);
 cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, int grid, cudaStream_t s);
 cudaError_t launch_beam(const TraceArgs& A, int fp_mode, int grid, cudaStream_t s);
 cudaError_t launch_detect(const TraceArgs& A, const EventsArgs& E, int fp_mode, int det, int grid,

@@ -12,8 +12,8 @@ cudaError_t launch_trace_f32(const TraceArgs& A, int det, int grid, cudaStream_t
 cudaError_t launch_trace_f64(const TraceArgs& A, int det, int grid, cudaStream_t s);
 int wave_threads_f32();
 int wave_threads_f64();
-cudaError_t blocks_per_sm_f32(int ns, int det, int bvk, int* blocks);
-cudaError_t blocks_per_sm_f64(int ns, int det, int bvk, int* blocks);
+cudaError_t blocks_per_sm_f32(int ns, int det, int bvk, int waves, int* blocks);
+cudaError_t blocks_per_sm_f64(int ns, int det, int bvk, int waves, int* blocks);
 cudaError_t launch_beam_f32(const TraceArgs& A, int grid, cudaStream_t s);
 cudaError_t launch_beam_f64(const TraceArgs& A, int grid, cudaStream_t s);
 cudaError_t launch_detect_f32(const TraceArgs& A, const EventsArgs& E, int det, int grid,
@@ -208,9 +208,9 @@ int trace_threads() { return 128; }
 
 int wave_threads(int fp_mode) { return fp_mode == MCV_FP32 ? wave_threads_f32() : wave_threads_f64(); }
 
-cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int* blocks) {
-  return fp_mode == MCV_FP32 ? blocks_per_sm_f32(ns, det, bvk, blocks)
-                             : blocks_per_sm_f64(ns, det, bvk, blocks);
+cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int waves, int* blocks) {
+  return fp_mode == MCV_FP32 ? blocks_per_sm_f32(ns, det, bvk, waves, blocks)
+                             : blocks_per_sm_f64(ns, det, bvk, waves, blocks);
 }
 
 cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, int grid, cudaStream_t s) {

@@ -127,7 +127,7 @@ mcv_status mcv_grad_noalloc(const mcv_sample* sample, const mcv_beam_params* bea
     A.tallies = hist->tallies;
     A.stop_on_zero = 1;
     int occ = 0;
-    e = mcv::trace_blocks_per_sm(fp, A.Sd.ns, A.Dd.kind, A.Sd.wide, &occ);
+    e = mcv::trace_blocks_per_sm(fp, A.Sd.ns, A.Dd.kind, A.Sd.wide, 1, &occ);
     if (e != cudaSuccess || occ < 1) occ = 1;
     e = mcv::launch_trace(A, fp, A.Dd.kind, grid_of(occ), s);
     if (e != cudaSuccess) return noalloc_fail(MCV_ECUDA, cudaGetErrorString(e));
