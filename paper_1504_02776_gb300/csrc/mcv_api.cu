@@ -551,21 +551,18 @@ mcv_status event_sink(const mcv_event_list* l, uint32_t tag, mcv::EvSink* out) {
 }
 
 int grid_for(mcv_ctx* ctx, int64_t items, int per_sm) {
-  const int64_t full = (int64_t)ctx->sm_count * per_sm;
-  const int64_t need = (items + mcv::trace_threads() - 1) / mcv::trace_threads();
-  int64_t g = need < full ? need : full;
-  return (int)(g < 1 ? 1 : g);
+  return mcv::lane_shape(items, ctx->sm_count, per_sm, mcv::trace_threads()).grid;
 }
 
-// resident blocks per SM of the kernel that traces A
-int trace_blocks(mcv_ctx* ctx, const mcv::TraceArgs& A, int fp, int det) {
+// the launch of the kernel that traces A
+mcv::LaunchShape shape_of(mcv_ctx* ctx, const mcv::TraceArgs& A, int fp, int det) {
   const int waves = mcv::uses_waves(A, det) ? 1 : 0;
   int& occ = ctx->occ[fp][ns_index(A.Sd.ns)][det][A.Sd.wide ? 1 : 0][waves];
   if (occ == 0) {
     cudaError_t e = mcv::trace_blocks_per_sm(fp, A.Sd.ns, det, A.Sd.wide, waves, &occ);
     if (e != cudaSuccess || occ < 1) occ = 1;
   }
-  return occ;
+  return mcv::trace_shape(A, fp, det, ctx->sm_count, occ);
 }
 
 PhiloxKeys philox_keys(uint32_t seed, uint32_t sim_id) {
@@ -833,9 +830,9 @@ mcv_status mcv_trace_sample(mcv_ctx* ctx, const mcv_sample* sample, const mcv_be
     if (e != cudaSuccess) return cuda_fail(e, "paper kernel launch");
     return MCV_OK;
   }
-  const int grid = grid_for(ctx, n, trace_blocks(ctx, A, fp, detk));
   cast_all(&A);
-  cudaError_t e = mcv::launch_trace(A, fp, detk, grid, static_cast<cudaStream_t>(stream));
+  cudaError_t e = mcv::launch_trace(A, fp, detk, shape_of(ctx, A, fp, detk),
+                                    static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "trace kernel launch");
   return MCV_OK;
 }
@@ -988,7 +985,7 @@ mcv_status mcv_grad(mcv_ctx* ctx, const mcv_sample* sample, const mcv_beam_param
     A.hist = hist->counts;
     A.tallies = hist->tallies;
     A.stop_on_zero = 1;
-    e = mcv::launch_trace(A, fp, A.Dd.kind, grid_for(ctx, n, trace_blocks(ctx, A, fp, A.Dd.kind)), s);
+    e = mcv::launch_trace(A, fp, A.Dd.kind, shape_of(ctx, A, fp, A.Dd.kind), s);
     if (e != cudaSuccess) return cuda_fail(e, "trace kernel launch");
   }
   return loss_and_adjoint(ctx, A, fp, hist->counts, target, scale_c, g_work, loss, dsqe, dsig, s);

@@ -1084,11 +1084,11 @@ namespace mcv {
 // ---- launchers, one set per real type -----------------------------------------------------
 // The fused waves with an event list are instantiated in translation units of their own
 // (mcv_fp32_ev.cu, mcv_fp64_ev.cu); these declare their entry points.
-cudaError_t launch_waves_ev_f32(const TraceArgs& A, int det, int grid, cudaStream_t s);
-cudaError_t launch_waves_ev_f64(const TraceArgs& A, int det, int grid, cudaStream_t s);
+cudaError_t launch_waves_ev_f32(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s);
+cudaError_t launch_waves_ev_f64(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s);
 template <typename R>
-cudaError_t launch_waves_ev(const TraceArgs& A, int det, int grid, cudaStream_t s) {
-  return sizeof(R) == 4 ? launch_waves_ev_f32(A, det, grid, s) : launch_waves_ev_f64(A, det, grid, s);
+cudaError_t launch_waves_ev(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s) {
+  return sizeof(R) == 4 ? launch_waves_ev_f32(A, det, L, s) : launch_waves_ev_f64(A, det, L, s);
 }
 
 template <typename R>
@@ -1107,67 +1107,67 @@ cudaError_t allow_wave_smem(const void* fn, bool batch) {
 }
 
 template <typename R, int NS, int DET, int KS>
-cudaError_t launch_trace_k(const TraceArgs& A, int grid, cudaStream_t s) {
+cudaError_t launch_trace_k(const TraceArgs& A, LaunchShape L, cudaStream_t s) {
   if (DET != MCV_DET_NONE && uses_waves(A, DET)) {
-    if (A.ev.count) return launch_waves_ev<R>(A, DET, grid, s);
+    if (A.ev.count) return launch_waves_ev<R>(A, DET, L, s);
     const size_t smem = wave_smem_bytes<R>(false, Dof_host<R>(A).max_tubes_row);
     cudaError_t e = allow_wave_smem<R>((const void*)wave_kernel<R, NS, DET, KS, false>, false);
     if (e != cudaSuccess) return e;
-    wave_kernel<R, NS, DET, KS, false><<<grid, WaveCfg<R>::threads, smem, s>>>(A);
+    wave_kernel<R, NS, DET, KS, false><<<L.grid, L.threads, smem, s>>>(A);
   } else {
-    trace_kernel<R, NS, DET, KS><<<grid, kThreads, 0, s>>>(A);
+    trace_kernel<R, NS, DET, KS><<<L.grid, L.threads, 0, s>>>(A);
   }
   return cudaGetLastError();
 }
 
 // the waves with an event list, over the shapes (used by the _ev translation units)
 template <typename R, int NS, int KS>
-cudaError_t launch_waves_ev_k(const TraceArgs& A, int det, int grid, cudaStream_t s) {
+cudaError_t launch_waves_ev_k(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s) {
   const size_t smem = wave_smem_bytes<R>(false, Dof_host<R>(A).max_tubes_row);
   const void* fn = det == MCV_DET_SURFACE ? (const void*)wave_kernel<R, NS, MCV_DET_SURFACE, KS, true>
                                           : (const void*)wave_kernel<R, NS, MCV_DET_TUBES, KS, true>;
   cudaError_t e = allow_wave_smem<R>(fn, false);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<TraceArgs*>(&A)};
-  return cudaLaunchKernel(fn, dim3(grid), dim3(WaveCfg<R>::threads), args, smem, s);
+  return cudaLaunchKernel(fn, dim3(L.grid), dim3(L.threads), args, smem, s);
 }
 
 template <typename R>
-cudaError_t launch_waves_ev_t(const TraceArgs& A, int det, int grid, cudaStream_t s) {
+cudaError_t launch_waves_ev_t(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s) {
   const bool all = A.Sd.wide;
   if (A.Sd.ns <= 1)
-    return all ? launch_waves_ev_k<R, 1, kKernelsAll>(A, det, grid, s)
-               : launch_waves_ev_k<R, 1, kKernelsPowder>(A, det, grid, s);
+    return all ? launch_waves_ev_k<R, 1, kKernelsAll>(A, det, L, s)
+               : launch_waves_ev_k<R, 1, kKernelsPowder>(A, det, L, s);
   if (A.Sd.ns == 2)
-    return all ? launch_waves_ev_k<R, 2, kKernelsAll>(A, det, grid, s)
-               : launch_waves_ev_k<R, 2, kKernelsPowder>(A, det, grid, s);
-  return all ? launch_waves_ev_k<R, 4, kKernelsAll>(A, det, grid, s)
-             : launch_waves_ev_k<R, 4, kKernelsPowder>(A, det, grid, s);
+    return all ? launch_waves_ev_k<R, 2, kKernelsAll>(A, det, L, s)
+               : launch_waves_ev_k<R, 2, kKernelsPowder>(A, det, L, s);
+  return all ? launch_waves_ev_k<R, 4, kKernelsAll>(A, det, L, s)
+             : launch_waves_ev_k<R, 4, kKernelsPowder>(A, det, L, s);
 }
 
 template <typename R, int NS, int KS>
-cudaError_t launch_trace_nk(const TraceArgs& A, int det, int grid, cudaStream_t s) {
+cudaError_t launch_trace_nk(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s) {
   switch (det) {
     case MCV_DET_SURFACE:
-      return launch_trace_k<R, NS, MCV_DET_SURFACE, KS>(A, grid, s);
+      return launch_trace_k<R, NS, MCV_DET_SURFACE, KS>(A, L, s);
     case MCV_DET_TUBES:
-      return launch_trace_k<R, NS, MCV_DET_TUBES, KS>(A, grid, s);
+      return launch_trace_k<R, NS, MCV_DET_TUBES, KS>(A, L, s);
     default:
-      return launch_trace_k<R, NS, MCV_DET_NONE, KS>(A, grid, s);
+      return launch_trace_k<R, NS, MCV_DET_NONE, KS>(A, L, s);
   }
 }
 
 template <typename R, int NS>
-cudaError_t launch_trace_ns(const TraceArgs& A, int det, int grid, cudaStream_t s) {
-  if (A.Sd.wide) return launch_trace_nk<R, NS, kKernelsAll>(A, det, grid, s);
-  return launch_trace_nk<R, NS, kKernelsPowder>(A, det, grid, s);
+cudaError_t launch_trace_ns(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s) {
+  if (A.Sd.wide) return launch_trace_nk<R, NS, kKernelsAll>(A, det, L, s);
+  return launch_trace_nk<R, NS, kKernelsPowder>(A, det, L, s);
 }
 
 template <typename R>
-cudaError_t launch_trace_t(const TraceArgs& A, int det, int grid, cudaStream_t s) {
-  if (A.Sd.ns <= 1) return launch_trace_ns<R, 1>(A, det, grid, s);
-  if (A.Sd.ns == 2) return launch_trace_ns<R, 2>(A, det, grid, s);
-  return launch_trace_ns<R, 4>(A, det, grid, s);
+cudaError_t launch_trace_t(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s) {
+  if (A.Sd.ns <= 1) return launch_trace_ns<R, 1>(A, det, L, s);
+  if (A.Sd.ns == 2) return launch_trace_ns<R, 2>(A, det, L, s);
+  return launch_trace_ns<R, 4>(A, det, L, s);
 }
 
 // the kernel that launch_trace launches for this shape: the waves, or one neutron per lane (a
@@ -1331,8 +1331,9 @@ cudaError_t launch_paper_t(const TraceArgs& A, int det, int grid, cudaStream_t s
 
 // defines the fused-trace entry points of one real type (mcv_fp32.cu / mcv_fp64.cu)
 #define MCV_DEFINE_TRACE_ENTRY_POINTS(R, SUFFIX)                                            \
-  cudaError_t launch_trace_##SUFFIX(const TraceArgs& A, int det, int grid, cudaStream_t s) { \
-    return launch_trace_t<R>(A, det, grid, s);                                              \
+  cudaError_t launch_trace_##SUFFIX(const TraceArgs& A, int det, LaunchShape L,             \
+                                    cudaStream_t s) {                                       \
+    return launch_trace_t<R>(A, det, L, s);                                                 \
   }                                                                                         \
   int wave_threads_##SUFFIX() { return WaveCfg<R>::threads; }                               \
   cudaError_t blocks_per_sm_##SUFFIX(int ns, int det, int bvk, int waves, int* blocks) {    \
@@ -1341,8 +1342,9 @@ cudaError_t launch_paper_t(const TraceArgs& A, int det, int grid, cudaStream_t s
 
 // the fused waves with an event list (mcv_fp32_ev.cu / mcv_fp64_ev.cu)
 #define MCV_DEFINE_EVENT_ENTRY_POINTS(R, SUFFIX)                                            \
-  cudaError_t launch_waves_ev_##SUFFIX(const TraceArgs& A, int det, int grid, cudaStream_t s) { \
-    return launch_waves_ev_t<R>(A, det, grid, s);                                           \
+  cudaError_t launch_waves_ev_##SUFFIX(const TraceArgs& A, int det, LaunchShape L,          \
+                                       cudaStream_t s) {                                    \
+    return launch_waves_ev_t<R>(A, det, L, s);                                              \
   }
 
 // the source, detector and adjoint entry points (mcv_fp32_aux.cu / mcv_fp64_aux.cu)

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "mcv_params.h"
+#include "mcv_shape.h"
 
 namespace mcv {
 
@@ -28,7 +29,12 @@ int trace_threads();
 int wave_threads(int fp_mode);
 // resident blocks per SM of the kernel launch_trace launches; waves: uses_waves
 cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int waves, int* blocks);
-cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, int grid, cudaStream_t s);
+// the launch that fills a GPU of `sms` SMs with A's n neutrons
+inline LaunchShape trace_shape(const TraceArgs& A, int fp_mode, int det, int sms, int blocks_per_sm) {
+  return uses_waves(A, det) ? wave_shape(A.n, sms, blocks_per_sm, wave_threads(fp_mode))
+                            : lane_shape(A.n, sms, blocks_per_sm, trace_threads());
+}
+cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, LaunchShape L, cudaStream_t s);
 cudaError_t launch_beam(const TraceArgs& A, int fp_mode, int grid, cudaStream_t s);
 cudaError_t launch_detect(const TraceArgs& A, const EventsArgs& E, int fp_mode, int det, int grid,
                           cudaStream_t s);

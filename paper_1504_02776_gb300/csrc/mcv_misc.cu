@@ -8,8 +8,8 @@
 
 namespace mcv {
 
-cudaError_t launch_trace_f32(const TraceArgs& A, int det, int grid, cudaStream_t s);
-cudaError_t launch_trace_f64(const TraceArgs& A, int det, int grid, cudaStream_t s);
+cudaError_t launch_trace_f32(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s);
+cudaError_t launch_trace_f64(const TraceArgs& A, int det, LaunchShape L, cudaStream_t s);
 int wave_threads_f32();
 int wave_threads_f64();
 cudaError_t blocks_per_sm_f32(int ns, int det, int bvk, int waves, int* blocks);
@@ -213,8 +213,8 @@ cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int waves
                              : blocks_per_sm_f64(ns, det, bvk, waves, blocks);
 }
 
-cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, int grid, cudaStream_t s) {
-  return fp_mode == MCV_FP32 ? launch_trace_f32(A, det, grid, s) : launch_trace_f64(A, det, grid, s);
+cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, LaunchShape L, cudaStream_t s) {
+  return fp_mode == MCV_FP32 ? launch_trace_f32(A, det, L, s) : launch_trace_f64(A, det, L, s);
 }
 
 cudaError_t launch_beam(const TraceArgs& A, int fp_mode, int grid, cudaStream_t s) {

@@ -115,13 +115,6 @@ mcv_status mcv_grad_noalloc(const mcv_sample* sample, const mcv_beam_params* bea
   A.err = reinterpret_cast<int*>(scratch);
   A.gs = grad_scatterer;
   const int fp = sample->fp_mode;
-  const int threads = mcv::trace_threads();
-  auto grid_of = [&](int per_sm) {
-    const int64_t full = (int64_t)sms * per_sm;
-    const int64_t need = (n + threads - 1) / threads;
-    const int64_t gsz = need < full ? need : full;
-    return (int)(gsz < 1 ? 1 : gsz);
-  };
   if (n > 0) {
     A.hist = hist->counts;
     A.tallies = hist->tallies;
@@ -129,7 +122,7 @@ mcv_status mcv_grad_noalloc(const mcv_sample* sample, const mcv_beam_params* bea
     int occ = 0;
     e = mcv::trace_blocks_per_sm(fp, A.Sd.ns, A.Dd.kind, A.Sd.wide, 1, &occ);
     if (e != cudaSuccess || occ < 1) occ = 1;
-    e = mcv::launch_trace(A, fp, A.Dd.kind, grid_of(occ), s);
+    e = mcv::launch_trace(A, fp, A.Dd.kind, mcv::trace_shape(A, fp, A.Dd.kind, sms, occ), s);
     if (e != cudaSuccess) return noalloc_fail(MCV_ECUDA, cudaGetErrorString(e));
   }
   e = mcv::launch_chi2(hist->counts, target, scale_c, A.Dd.n_bins, g, loss,
@@ -145,7 +138,7 @@ mcv_status mcv_grad_noalloc(const mcv_sample* sample, const mcv_beam_params* bea
     int occ_a = 0;
     e = mcv::adjoint_blocks_per_sm(fp, A.Sd.ns, A.Dd.kind, A.Sd.wide, &occ_a);
     if (e != cudaSuccess || occ_a < 1) occ_a = 1;
-    e = mcv::launch_adjoint(A, fp, A.Dd.kind, grid_of(occ_a), s);
+    e = mcv::launch_adjoint(A, fp, A.Dd.kind, mcv::lane_shape(n, sms, occ_a, mcv::trace_threads()).grid, s);
     if (e != cudaSuccess) return noalloc_fail(MCV_ECUDA, cudaGetErrorString(e));
   }
   return MCV_OK;

@@ -1,0 +1,16 @@
+// Prints "n sms blocks_per_sm threads -> grid threads" of csrc/mcv_shape.h for the counts given on
+// the command line, one line each for the waves ("w") and for one neutron per lane ("l").
+#include <cstdio>
+#include <cstdlib>
+
+#include "mcv_shape.h"
+
+int main(int argc, char** argv) {
+  const int sms = std::atoi(argv[1]), per_sm = std::atoi(argv[2]), threads = std::atoi(argv[3]);
+  for (int i = 4; i < argc; ++i) {
+    const long long n = std::atoll(argv[i]);
+    const mcv::LaunchShape w = mcv::wave_shape(n, sms, per_sm, threads);
+    const mcv::LaunchShape l = mcv::lane_shape(n, sms, per_sm, threads);
+    std::printf("w %lld %d %d\nl %lld %d %d\n", n, w.grid, w.threads, n, l.grid, l.threads);
+  }
+}
