@@ -1,5 +1,6 @@
-// Prints "n sms blocks_per_sm threads -> grid threads" of csrc/mcv_shape.h for the counts given on
-// the command line, one line each for the waves ("w") and for one neutron per lane ("l").
+// Prints "n grid threads" of csrc/mcv_shape.h for the counts given on the command line after SMs,
+// blocks per SM, threads and least warps, a line each for the waves ("w") and for one neutron per
+// lane ("l").
 #include <cstdio>
 #include <cstdlib>
 
@@ -7,9 +8,10 @@
 
 int main(int argc, char** argv) {
   const int sms = std::atoi(argv[1]), per_sm = std::atoi(argv[2]), threads = std::atoi(argv[3]);
-  for (int i = 4; i < argc; ++i) {
+  const int least = std::atoi(argv[4]);
+  for (int i = 5; i < argc; ++i) {
     const long long n = std::atoll(argv[i]);
-    const mcv::LaunchShape w = mcv::wave_shape(n, sms, per_sm, threads);
+    const mcv::LaunchShape w = mcv::wave_shape(n, sms, per_sm, threads, least);
     const mcv::LaunchShape l = mcv::lane_shape(n, sms, per_sm, threads);
     std::printf("w %lld %d %d\nl %lld %d %d\n", n, w.grid, w.threads, n, l.grid, l.threads);
   }

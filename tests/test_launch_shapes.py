@@ -11,8 +11,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_1504_02776_gb300", "csrc")
 
 
-@pytest.mark.parametrize("sms,per_sm,threads", [(152, 1, 640), (152, 1, 384), (7, 2, 128)])
-def test_shapes_fill_warps_and_sms(tmp_path, sms, per_sm, threads):
+@pytest.mark.parametrize("sms,per_sm,threads,least", [(152, 1, 640, 4), (152, 1, 384, 1), (7, 2, 128, 1)])
+def test_shapes_fill_warps_and_sms(tmp_path, sms, per_sm, threads, least):
     exe = str(tmp_path / "launch_shape_check")
     subprocess.run(["g++", "-O2", "-std=gnu++17", "-I" + CSRC, "-x", "c++",
                     os.path.join(HERE, "launch_shape_check.cpp"), "-o", exe], check=True)
@@ -20,7 +20,7 @@ def test_shapes_fill_warps_and_sms(tmp_path, sms, per_sm, threads):
     full = 32 * room * (threads // 32)
     counts = [1, 31, 32, 33, 1000, 3001, 10000, 32 * room, 32 * room + 1, 30011, 60000, full - 31,
               full, full + 1, 100003, 10 ** 8, 2 ** 40]
-    out = subprocess.run([exe, str(sms), str(per_sm), str(threads)] + [str(n) for n in counts],
+    out = subprocess.run([exe, str(sms), str(per_sm), str(threads), str(least)] + [str(n) for n in counts],
                          check=True, capture_output=True, text=True).stdout
     for line in out.splitlines():
         kind, n, grid, block = line[0], *map(int, line[2:].split())
@@ -34,4 +34,4 @@ def test_shapes_fill_warps_and_sms(tmp_path, sms, per_sm, threads):
             continue
         warps, batches = lanes // 32, (n + 31) // 32
         assert batches <= warps < batches + block // 32, line  # no block without a batch
-        assert grid >= min(batches, (room + 1) // 2), line
+        assert grid >= min((batches + least - 1) // least, (room + 1) // 2), line
