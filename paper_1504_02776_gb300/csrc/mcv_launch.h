@@ -31,9 +31,10 @@ int wave_threads(int fp_mode);
 cudaError_t trace_blocks_per_sm(int fp_mode, int ns, int det, int bvk, int waves, int* blocks);
 // the launch that fills a GPU of `sms` SMs with A's n neutrons
 inline LaunchShape trace_shape(const TraceArgs& A, int fp_mode, int det, int sms, int blocks_per_sm) {
-  return uses_waves(A, det) ? wave_shape(A.n, sms, blocks_per_sm, wave_threads(fp_mode),
-                                         fp_mode == MCV_FP32 ? 4 : 1)
-                            : lane_shape(A.n, sms, blocks_per_sm, trace_threads());
+  if (uses_waves(A, det))
+    return wave_shape(A.n, sms, blocks_per_sm, wave_threads(fp_mode), fp_mode == MCV_FP32 ? 4 : 1);
+  return det != MCV_DET_NONE ? chain_shape(A.n, sms, blocks_per_sm, trace_threads())
+                             : lane_shape(A.n, sms, blocks_per_sm, trace_threads());
 }
 cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, LaunchShape L, cudaStream_t s);
 cudaError_t launch_beam(const TraceArgs& A, int fp_mode, int grid, cudaStream_t s);

@@ -1,6 +1,6 @@
 // Prints "n grid threads" of csrc/mcv_shape.h for the counts given on the command line after SMs,
-// blocks per SM, threads and least warps, a line each for the waves ("w") and for one neutron per
-// lane ("l").
+// blocks per SM, threads and least warps, a line each for the waves ("w"), for one item per lane
+// ("l") and for refilled lanes ("c").
 #include <cstdio>
 #include <cstdlib>
 
@@ -13,6 +13,8 @@ int main(int argc, char** argv) {
     const long long n = std::atoll(argv[i]);
     const mcv::LaunchShape w = mcv::wave_shape(n, sms, per_sm, threads, least);
     const mcv::LaunchShape l = mcv::lane_shape(n, sms, per_sm, threads);
-    std::printf("w %lld %d %d\nl %lld %d %d\n", n, w.grid, w.threads, n, l.grid, l.threads);
+    const mcv::LaunchShape c = mcv::chain_shape(n, sms, per_sm, threads);
+    std::printf("w %lld %d %d\nl %lld %d %d\nc %lld %d %d\n", n, w.grid, w.threads, n, l.grid,
+                l.threads, n, c.grid, c.threads);
   }
 }

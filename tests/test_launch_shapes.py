@@ -29,6 +29,10 @@ def test_shapes_fill_warps_and_sms(tmp_path, sms, per_sm, threads, least):
         if kind == "l":
             assert lanes >= n or grid == room, line
             continue
+        if kind == "c":
+            assert grid == room or (grid >= min(sms, (n + threads - 1) // threads)
+                                    and 2 * lanes >= n), line
+            continue
         if n >= full:
             assert lanes == full, line
             continue
