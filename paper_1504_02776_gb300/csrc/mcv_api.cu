@@ -877,7 +877,7 @@ mcv_status mcv_detect(mcv_ctx* ctx, const mcv_detector* det, int fp_mode,
   mcv::EventsArgs E{nullptr, nullptr, nullptr, nullptr};
   if (events) E = mcv::EventsArgs{events->pixel, events->tof, events->w_det, events->bin};
   cast_all(&A);
-  cudaError_t e = mcv::launch_detect(A, E, fp_mode, A.Dd.kind, grid_for(ctx, packets->n, 8),
+  cudaError_t e = mcv::launch_detect(A, E, fp_mode, A.Dd.kind, ctx->sm_count,
                                      static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "detect kernel launch");
   return MCV_OK;

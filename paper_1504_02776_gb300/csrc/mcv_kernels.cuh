@@ -837,64 +837,83 @@ __device__ __forceinline__ void detect_slot(const TraceArgs& A, const EventsArgs
 }
 
 // Detector system on stored packets.  A run's slots are mostly empty (a neutron that misses the
-// sample fills one of max_orders + 1), so each warp reads the orders of 4 x 32 slots at a time
-// and queues the packets to be detected; batches of 32 of them are traced together.  With a
-// slot per lane 5.7 of 32 lanes traced, and every trace waited for its own loads.  The unfused
-// chain of 5e5 neutrons (FP32 powder, 3e6 slots): 280 -> 235 us, of which this kernel was 138.
+// sample fills one of max_orders + 1), so a block reads the orders of `rows` x 128 slots at a time
+// and queues the packets to be detected; its warps then trace full batches of 32 of them.  With
+// a slot per lane 5.7 of 32 lanes traced, and every trace waited for its own loads.  The queue is
+// the block's, so that the packets of a dense list are traced by all its warps at once, and a
+// short list is read by as many blocks as it has 128 slots (rows: detect_shape).  Against a slot
+// per lane / a queue per warp that read 4 x 32 slots / this: dense list of 3e4 packets, FP64,
+// 44.0 / 68.8 / 33.8 us, of 1e5, FP32, 37.8 / 39.7 / 23.8; the 3e5 slots of a run, FP64,
+// 195 / 82.4 / 42.0, FP32, 85.6 / 48.4 / 27.6; the 3e6 of the unfused chain of 5e5 neutrons, FP32,
+// 280 / 233 / 233 for the whole chain.
+constexpr int kDetectRows = 4;
+
 template <typename R, int DET>
 __global__ void __launch_bounds__(kThreads) detect_kernel(const __grid_constant__ TraceArgs A,
-                                                          EventsArgs E) {
+                                                          EventsArgs E, int rows) {
   __shared__ R tu[2 * MCV_MAX_TUBES_PER_ROW];
-  __shared__ int64_t queues[kThreads / 32][kQueue];  // slot index x 8 + order
+  __shared__ int64_t queue[kDetectRows * kThreads + 32];  // slot index x 8 + order
+  __shared__ int found[kThreads / 32];
   stage_tubes<R, DET>(A, tu);
+  static_assert(kMaxOrders < 8, "an order fits the queue entry's low three bits");
   const unsigned kFull = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
-  int64_t* queue = queues[threadIdx.x >> 5];
   Acc<R> a_bs, a_det, a_over;
   Counts cnt;
-  int err = 0, qn = 0;
-  constexpr int kGroups = 4;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t groups = (A.n + 31) / 32;
-  const int64_t first = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  for (int64_t g0 = first * kGroups; g0 < groups; g0 += warps * kGroups) {
-    int order[kGroups];
+  int err = 0, qn = 0;  // qn: queued packets, the same in every thread (at most 31 here)
+  const int64_t chunk = (int64_t)rows * kThreads, stride = chunk * gridDim.x;
+  for (int64_t base = blockIdx.x * chunk; base < A.n; base += stride) {
+    int order[kDetectRows];
+    unsigned mask[kDetectRows];
 #pragma unroll
-    for (int k = 0; k < kGroups; ++k) {
-      const int64_t i = (g0 + k) * 32 + lane;
-      order[k] = i < A.n ? A.in_order[i] : -1;
+    for (int k = 0; k < kDetectRows; ++k) {
+      const int64_t i = base + k * kThreads + threadIdx.x;
+      order[k] = k < rows && i < A.n ? A.in_order[i] : -1;
     }
-    const bool last = g0 + warps * kGroups >= groups;  // drain the queue
-#pragma unroll 1
-    for (int k = 0; k < kGroups; ++k) {
-      const int64_t i = (g0 + k) * 32 + lane;
-      int o = order[0];
+    int mine = 0;
 #pragma unroll
-      for (int m = 1; m < kGroups; ++m) o = k == m ? order[m] : o;
-      if (o > kMaxOrders) {  // no packet of the library has such an order: flag it, skip it
+    for (int k = 0; k < kDetectRows; ++k) {
+      const int64_t i = base + k * kThreads + threadIdx.x;
+      if (order[k] > kMaxOrders) {  // no packet of the library has such an order: flag it, skip it
         err = 1;
-        o = -1;
+        order[k] = -1;
       }
-      if (o == 0) {
+      if (order[k] == 0) {
         a_bs.add(static_cast<const R*>(A.in_w)[i]);
         if (E.bin) E.bin[i] = -1;
         if (E.pixel) E.pixel[i] = -1;
         if (E.tof) E.tof[i] = 0.0;
         if (E.w_det) E.w_det[i] = 0.0;
       }
-      const unsigned mm = __ballot_sync(kFull, o > 0);
-      if (o > 0) queue[qn + __popc(mm & lt_mask)] = i * 8 + o;
-      qn += __popc(mm);
-      __syncwarp();
-      while (qn >= 32 || (last && k == kGroups - 1 && qn > 0)) {
-        const int take = qn < 32 ? qn : 32;
-        const int64_t e = lane < take ? queue[qn - take + lane] : -1;
-        qn -= take;
-        __syncwarp();
-        if (e >= 0) detect_slot<R, DET>(A, E, tu, e >> 3, (int)(e & 7), a_det, a_over, cnt, err);
-      }
+      mask[k] = __ballot_sync(kFull, order[k] > 0);
+      mine += __popc(mask[k]);
     }
+    if (lane == 0) found[warp] = mine;
+    __syncthreads();
+    int at = qn;
+    for (int w = 0; w < kThreads / 32; ++w) {
+      if (w < warp) at += found[w];
+      qn += found[w];
+    }
+#pragma unroll
+    for (int k = 0; k < kDetectRows; ++k) {
+      if (order[k] > 0)
+        queue[at + __popc(mask[k] & lt_mask)] = (base + k * kThreads + threadIdx.x) * 8 + order[k];
+      at += __popc(mask[k]);
+    }
+    __syncthreads();
+    // full batches from the queue's end; the remainder with the last slots
+    const int batches = base + stride >= A.n ? (qn + 31) / 32 : qn / 32;
+    for (int b = warp; b < batches; b += kThreads / 32) {
+      const int q = qn - 32 * (b + 1) + lane;
+      if (q >= 0) {
+        const int64_t e = queue[q];
+        detect_slot<R, DET>(A, E, tu, e >> 3, (int)(e & 7), a_det, a_over, cnt, err);
+      }
+      __syncwarp();
+    }
+    qn = max(0, qn - 32 * batches);
   }
   if (A.tallies) {
     const double v_bs = warp_sum(a_bs.value());
@@ -1254,12 +1273,13 @@ cudaError_t launch_beam_t(const TraceArgs& A, int grid, cudaStream_t s) {
 }
 
 template <typename R>
-cudaError_t launch_detect_t(const TraceArgs& A, const EventsArgs& E, int det, int grid,
+cudaError_t launch_detect_t(const TraceArgs& A, const EventsArgs& E, int det, int sms,
                             cudaStream_t s) {
+  const DetectShape L = detect_shape(A.n, sms, kThreads, kDetectRows);
   if (det == MCV_DET_SURFACE)
-    detect_kernel<R, MCV_DET_SURFACE><<<grid, kThreads, 0, s>>>(A, E);
+    detect_kernel<R, MCV_DET_SURFACE><<<L.grid, kThreads, 0, s>>>(A, E, L.rows);
   else
-    detect_kernel<R, MCV_DET_TUBES><<<grid, kThreads, 0, s>>>(A, E);
+    detect_kernel<R, MCV_DET_TUBES><<<L.grid, kThreads, 0, s>>>(A, E, L.rows);
   return cudaGetLastError();
 }
 
@@ -1353,8 +1373,8 @@ cudaError_t launch_paper_t(const TraceArgs& A, int det, int grid, cudaStream_t s
     return launch_beam_t<R>(A, grid, s);                                                    \
   }                                                                                         \
   cudaError_t launch_detect_##SUFFIX(const TraceArgs& A, const EventsArgs& E, int det,      \
-                                     int grid, cudaStream_t s) {                            \
-    return launch_detect_t<R>(A, E, det, grid, s);                                          \
+                                     int sms, cudaStream_t s) {                             \
+    return launch_detect_t<R>(A, E, det, sms, s);                                           \
   }                                                                                         \
   cudaError_t launch_adjoint_##SUFFIX(const TraceArgs& A, int det, int grid,                \
                                       cudaStream_t s) {                                     \

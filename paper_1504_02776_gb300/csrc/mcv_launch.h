@@ -38,7 +38,7 @@ inline LaunchShape trace_shape(const TraceArgs& A, int fp_mode, int det, int sms
 }
 cudaError_t launch_trace(const TraceArgs& A, int fp_mode, int det, LaunchShape L, cudaStream_t s);
 cudaError_t launch_beam(const TraceArgs& A, int fp_mode, int grid, cudaStream_t s);
-cudaError_t launch_detect(const TraceArgs& A, const EventsArgs& E, int fp_mode, int det, int grid,
+cudaError_t launch_detect(const TraceArgs& A, const EventsArgs& E, int fp_mode, int det, int sms,
                           cudaStream_t s);
 cudaError_t launch_zero(double* p, int64_t n, int grid, cudaStream_t s);
 // chi-squared loss into *loss (accumulated); g (optional) receives dchi2/dI per bin; err

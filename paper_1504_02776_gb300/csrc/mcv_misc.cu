@@ -16,9 +16,9 @@ cudaError_t blocks_per_sm_f32(int ns, int det, int bvk, int waves, int* blocks);
 cudaError_t blocks_per_sm_f64(int ns, int det, int bvk, int waves, int* blocks);
 cudaError_t launch_beam_f32(const TraceArgs& A, int grid, cudaStream_t s);
 cudaError_t launch_beam_f64(const TraceArgs& A, int grid, cudaStream_t s);
-cudaError_t launch_detect_f32(const TraceArgs& A, const EventsArgs& E, int det, int grid,
+cudaError_t launch_detect_f32(const TraceArgs& A, const EventsArgs& E, int det, int sms,
                               cudaStream_t s);
-cudaError_t launch_detect_f64(const TraceArgs& A, const EventsArgs& E, int det, int grid,
+cudaError_t launch_detect_f64(const TraceArgs& A, const EventsArgs& E, int det, int sms,
                               cudaStream_t s);
 cudaError_t launch_adjoint_f32(const TraceArgs& A, int det, int grid, cudaStream_t s);
 cudaError_t launch_adjoint_f64(const TraceArgs& A, int det, int grid, cudaStream_t s);
@@ -221,10 +221,10 @@ cudaError_t launch_beam(const TraceArgs& A, int fp_mode, int grid, cudaStream_t 
   return fp_mode == MCV_FP32 ? launch_beam_f32(A, grid, s) : launch_beam_f64(A, grid, s);
 }
 
-cudaError_t launch_detect(const TraceArgs& A, const EventsArgs& E, int fp_mode, int det, int grid,
+cudaError_t launch_detect(const TraceArgs& A, const EventsArgs& E, int fp_mode, int det, int sms,
                           cudaStream_t s) {
-  return fp_mode == MCV_FP32 ? launch_detect_f32(A, E, det, grid, s)
-                             : launch_detect_f64(A, E, det, grid, s);
+  return fp_mode == MCV_FP32 ? launch_detect_f32(A, E, det, sms, s)
+                             : launch_detect_f64(A, E, det, sms, s);
 }
 
 cudaError_t launch_adjoint(const TraceArgs& A, int fp_mode, int det, int grid, cudaStream_t s) {

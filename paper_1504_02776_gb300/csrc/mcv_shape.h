@@ -44,4 +44,19 @@ inline LaunchShape chain_shape(int64_t n, int sms, int blocks_per_sm, int thread
   return one.grid <= sms ? one : (two.grid < sms ? LaunchShape{sms, threads} : two);
 }
 
+// Stored packets (detect_kernel): up to 8 blocks per SM, each of which reads `rows` x `threads`
+// slots at a time: max_rows of them once that leaves every SM two blocks, fewer where the list is
+// shorter.
+struct DetectShape {
+  int grid, rows;
+};
+
+inline DetectShape detect_shape(int64_t n, int sms, int threads, int max_rows) {
+  const int64_t room = (int64_t)sms * 8;
+  int64_t rows = n / ((int64_t)sms * 2 * threads);
+  rows = rows < 1 ? 1 : (rows < max_rows ? rows : max_rows);
+  const int64_t need = n < 1 ? 1 : (n + rows * threads - 1) / (rows * threads);
+  return DetectShape{(int)(need < room ? need : room), (int)rows};
+}
+
 }  // namespace mcv

@@ -1,6 +1,6 @@
 // Prints "n grid threads" of csrc/mcv_shape.h for the counts given on the command line after SMs,
 // blocks per SM, threads and least warps, a line each for the waves ("w"), for one item per lane
-// ("l") and for refilled lanes ("c").
+// ("l") and for refilled lanes ("c"), and "n grid rows" for stored packets ("d").
 #include <cstdio>
 #include <cstdlib>
 
@@ -16,5 +16,7 @@ int main(int argc, char** argv) {
     const mcv::LaunchShape c = mcv::chain_shape(n, sms, per_sm, threads);
     std::printf("w %lld %d %d\nl %lld %d %d\nc %lld %d %d\n", n, w.grid, w.threads, n, l.grid,
                 l.threads, n, c.grid, c.threads);
+    const mcv::DetectShape d = mcv::detect_shape(n, sms, threads, 4);
+    std::printf("d %lld %d %d\n", n, d.grid, d.rows);
   }
 }

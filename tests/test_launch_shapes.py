@@ -24,6 +24,11 @@ def test_shapes_fill_warps_and_sms(tmp_path, sms, per_sm, threads, least):
                          check=True, capture_output=True, text=True).stdout
     for line in out.splitlines():
         kind, n, grid, block = line[0], *map(int, line[2:].split())
+        if kind == "d":  # block: the rows; no idle block, and no longer rows than leave two per SM
+            assert 1 <= block <= 4 and 1 <= grid <= 8 * sms, line
+            assert grid == 8 * sms or (grid - 1) * block * threads < n <= grid * block * threads, line
+            assert block == 1 or n >= 2 * sms * threads * block, line
+            continue
         assert 1 <= grid <= room and 32 <= block <= threads and block % 32 == 0, line
         lanes = grid * block
         if kind == "l":
