@@ -29,7 +29,7 @@ struct mcv_ctx {
 namespace mcv {
 namespace host {
 
-constexpr int64_t kMaxNeutrons = (int64_t)1 << 40;
+using mcv::kMaxNeutrons;
 
 mcv_status fail(mcv_status st, const std::string& msg);
 mcv_status cuda_fail(cudaError_t e, const char* where);

@@ -191,6 +191,7 @@ struct QPacket<double> {
 struct QFoot {
   uint32_t a, b, c, d, i_lo;
 };
+static_assert(kMaxNeutrons <= (int64_t)1 << 43, "an index fits QFoot's 32 + 11 bits (and QPacket's 32 + 24)");
 
 template <typename R>
 constexpr size_t queue_bytes() {  // of one warp
@@ -219,14 +220,14 @@ struct CountMisses {
   __device__ __forceinline__ void operator()() const {}
 };
 template <typename R, int NS, bool DROP, class Job, class Src, class Miss = CountMisses>
-__device__ __forceinline__ uint32_t source_stage(const TraceArgs& A, const Job& job, int need,
+__device__ __forceinline__ uint64_t source_stage(const TraceArgs& A, const Job& job, int need,
                                                  int64_t& next, int64_t& hi, Src& src,
                                                  SourceQueues<R>& q, const Miss& on_miss = Miss()) {
   const SampleP<R>& S = job.S();
   const unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
-  uint32_t missed = 0;
+  uint64_t missed = 0;
   while (q.hq_n < need && (q.fq_n > 0 || next < hi || src.more(&next, &hi))) {
     if (q.fq_n < 32 && (next < hi || src.more(&next, &hi))) {
       const int64_t i = next + lane;
@@ -290,7 +291,7 @@ __device__ __forceinline__ uint32_t source_stage(const TraceArgs& A, const Job& 
     __syncwarp();
   }
   // a neutron of weight 1 counts at the beam stop unless it is lighter than min_prob
-  return Miss::kPerLane || R(1) < S.min_prob ? 0u : missed;
+  return Miss::kPerLane || R(1) < S.min_prob ? 0 : missed;
 }
 
 // a queued neutron as a packet of order 0; returns its id
@@ -331,10 +332,12 @@ struct BatchWarp {
   int home, v;
 };
 
-// A warp's counts, updated by its lane 0.
+// A warp's counts, updated by its lane 0.  A warp can be handed all of a simulation's neutrons, with
+// up to kMaxOrders packets each: beyond 32 bits.
 struct WarpCounts {
-  uint32_t beam, hit, emit, miss, det, over;
+  uint64_t beam, hit, emit, miss, det, over;
 };
+static_assert(kMaxNeutrons <= INT64_MAX / kMaxOrders, "a warp's counts fit 64 bits");
 
 // a thread's weight sums
 template <typename R>
@@ -560,7 +563,7 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
     const int n_idle = __popc(idle);
     // ---- source stage
     const LaneMisses<R, P> on_miss{pol};
-    const uint32_t n_beam = source_stage<R, NS, true>(A, job, n_idle, next, hi, src, q, on_miss);
+    const uint64_t n_beam = source_stage<R, NS, true>(A, job, n_idle, next, hi, src, q, on_miss);
     const int take = min(n_idle, q.hq_n);
     if (!L.active) {
       const int r = __popc(idle & lt_mask);

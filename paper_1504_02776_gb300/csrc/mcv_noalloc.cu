@@ -78,7 +78,7 @@ mcv_status mcv_grad_noalloc(const mcv_sample* sample, const mcv_beam_params* bea
     return noalloc_fail(MCV_EINVAL, "the histogram has " + std::to_string(A.Dd.n_bins) +
                                         " bins; mcv_grad_noalloc holds at most " +
                                         std::to_string(kMaxBins));
-  if (n < 0 || n > ((int64_t)1 << 40) || first_id < 0 || first_id > (((int64_t)1 << 62) - n))
+  if (n < 0 || n > mcv::kMaxNeutrons || first_id < 0 || first_id > (((int64_t)1 << 62) - n))
     return noalloc_fail(MCV_EINVAL, "bad neutron range");
   if (!target || !loss || !dsig || !hist || !hist->counts)
     return noalloc_fail(MCV_EINVAL, "needs target, hist->counts, loss and dsig");

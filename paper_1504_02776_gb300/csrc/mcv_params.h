@@ -20,6 +20,9 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr double kMeVPerV2 = 0.5 * kNeutronMass / (kElemCharge * 1e-3);
 constexpr double kKPerV = kNeutronMass / kHbar * 1e-10;
 
+// largest number of neutrons of a call (or of one simulation of a batch)
+constexpr int64_t kMaxNeutrons = (int64_t)1 << 40;
+
 template <typename R>
 struct BeamP {
   R ei, rel, div, width, height, z0, l1;
