@@ -379,8 +379,11 @@ mcv_status mcv_adjoint(mcv_ctx* ctx, const mcv_sample* sample, const mcv_beam_pa
  * warp starts at a simulation of its own (warps spread in proportion to the neutron counts),
  * takes that simulation's items until its queue is empty, then helps with the others, so
  * uneven simulations keep every SM busy to the end.  Each neutron's history
- * and arithmetic are those of mcv_trace_sample with the same simulation's arguments; only
- * the order of the FP64 histogram additions differs.
+ * is that of mcv_trace_sample with the same simulation's arguments.  In FP64 its arithmetic is
+ * too: only the order of the FP64 histogram additions differs.  In FP32 so it is for one-scatterer
+ * powder samples (isotropic and S(Q,E) kernels); with others the two kernels round a tube chord
+ * next to the tube's edge differently (and the dispersion kernel's last bits): 1 to 2 in 1000
+ * bins differ, the histograms by 1e-8 to 2e-7 of their sum.
  *
  * One simulation of a batch.  sample, beam: as mcv_trace_sample (sample->fp_mode must be
  * the batch's fp_mode); ids first_id..first_id+n-1 of the stream (seed, sim_id);

@@ -384,10 +384,10 @@ __device__ __forceinline__ bool make_beam(const BeamP<R>& B, const Rng& rng, Ray
 // ---- geometry ----------------------------------------------------------------------------
 // Line r + s d inside the infinite cylinder x^2 + z^2 < rad^2 (axis y): closest-approach
 // form, squared axis distance (r x d)^2 / a with a = dx^2 + dz^2.
-template <typename R, bool NORM = false>
+template <typename R, bool SWAP = false>
 __device__ __forceinline__ bool cyl_span(R rad, R x, R z, R dx, R dz, R* s1, R* s2) {
   using M = Mth<R>;
-  const R a = NORM ? M::norm2(dx, dz) : dx * dx + dz * dz;
+  const R a = SWAP ? M::norm2(dz, dx) : M::norm2(dx, dz);
   if (M::is_zero(a)) {
     if (x * x + z * z < rad * rad) {
       *s1 = -M::inf();
@@ -1371,10 +1371,10 @@ struct Hit {
 };
 
 // larger root of the ray with the origin-centred cylinder (the ray starts inside it)
-template <typename R, bool NORM>
+template <typename R, bool SWAP>
 __device__ __forceinline__ bool exit_cyl(R rad, const Ray<R>& n, R* s) {
   R s1, s2;
-  if (!cyl_span<R, NORM>(rad, n.x, n.z, n.dx, n.dz, &s1, &s2)) return false;
+  if (!cyl_span<R, SWAP>(rad, n.x, n.z, n.dx, n.dz, &s1, &s2)) return false;
   if (!Mth<R>::positive(s2) || !Mth<R>::lt(s2, Mth<R>::inf())) return false;
   *s = s2;
   return true;
@@ -1382,9 +1382,10 @@ __device__ __forceinline__ bool exit_cyl(R rad, const Ray<R>& n, R* s) {
 
 // Chord of a vertical tube (axis through R (ux, uz)) in coordinates along / across the
 // tube direction, so the large distance R cancels once.
-template <typename R, bool NORM = false, int FORM = 0>
+// SWAP, QUOTIENT (FP32): see detect().
+template <typename R, bool SWAP = false, bool QUOTIENT = false>
 __device__ __forceinline__ bool tube_span(R Rad, R ux, R uz, R rt, const Ray<R>& n, R* s1, R* s2) {
-  const R a = NORM ? Mth<R>::norm2(n.dx, n.dz) : n.dx * n.dx + n.dz * n.dz;
+  const R a = SWAP ? Mth<R>::norm2(n.dz, n.dx) : Mth<R>::norm2(n.dx, n.dz);
   if (Mth<R>::is_zero(a)) return false;
   const typename Mth<R>::Rcp ra = Mth<R>::rcp(a);
   const R o_rad = n.x * ux + n.z * uz - Rad;
@@ -1394,18 +1395,12 @@ __device__ __forceinline__ bool tube_span(R Rad, R ux, R uz, R rt, const Ray<R>&
   const R tc = Mth<R>::divr(-(o_rad * d_rad + o_tan * d_tan), ra);
   const R cr = o_rad * d_tan - o_tan * d_rad;
   R g;
-  if constexpr (sizeof(R) == 4 && FORM != 0) {
-    // a chord next to the tube's edge is its rounding: held in the kernel's form
-    if constexpr (FORM == 1) {
-      g = __fmaf_rn(rt, rt, -(cr * cr / a));
-    } else {
-      float ia;
-      asm("rcp.approx.f32 %0, %1;" : "=f"(ia) : "f"(a));
-      g = __fmaf_rn(-__fmul_rn(cr, cr), ia, __fmul_rn(rt, rt));
-    }
-  } else {
+  if constexpr (sizeof(R) == 8)
     g = rt * rt - Mth<R>::divr(cr * cr, ra);
-  }
+  else if constexpr (QUOTIENT)
+    g = __fmaf_rn(rt, rt, -(cr * cr / a));
+  else
+    g = __fmaf_rn(-__fmul_rn(cr, cr), 1.0f / a, __fmul_rn(rt, rt));
   if (!Mth<R>::positive(g)) return false;
   const R half = Mth<R>::sqrt(Mth<R>::divr(g, ra));
   *s1 = tc - half;
@@ -1429,7 +1424,7 @@ __device__ __forceinline__ int64_t tof_bin<float>(const TofWin& W, const Tof<flo
   return (int64_t)fb;
 }
 
-template <typename R, bool NORM>
+template <typename R, bool SWAP>
 __device__ __forceinline__ Hit<R> detect_surface(const DetP<R>& D, const TofWin& W,
                                                  const Ray<R>& n) {
   using M = Mth<R>;
@@ -1440,7 +1435,7 @@ __device__ __forceinline__ Hit<R> detect_surface(const DetP<R>& D, const TofWin&
   h.w_det = R(0);
   h.pabs = R(0);
   R s;
-  if (!exit_cyl<R, NORM>((R)D.radius, n, &s)) return h;
+  if (!exit_cyl<R, SWAP>((R)D.radius, n, &s)) return h;
   const R yh = n.y + s * n.dy;
   const R half = (R)D.half_h;
   if (M::lt(yh, -half) || M::le(half, yh)) return h;
@@ -1483,13 +1478,13 @@ __device__ __forceinline__ bool det_surely_misses(const DetP<R>& D, const Ray<R>
 // Where a packet meets the tube rows: the row at its crossing of the tube-centre circle and
 // the tube g nearest to that crossing (candidates g - 1, g, g + 1).  False: it meets no row
 // or lies outside the rows' arc (no candidate tube), i.e. it misses the detector.
-template <typename R, bool NORM = false>
+template <typename R, bool SWAP = false>
 __device__ __forceinline__ bool tubes_locate(const DetP<R>& D, const Ray<R>& n, int* row_out,
                                              int* g_out) {
   using M = Mth<R>;
   const R Rad = (R)D.radius;
   R sR;
-  if (!exit_cyl<R, NORM>(Rad, n, &sR)) return false;
+  if (!exit_cyl<R, SWAP>(Rad, n, &sR)) return false;
   const R Px = n.x + sR * n.dx, Py = n.y + sR * n.dy, Pz = n.z + sR * n.dz;
   int row = -1;
 #pragma unroll
@@ -1517,7 +1512,7 @@ __device__ __forceinline__ bool tubes_locate(const DetP<R>& D, const Ray<R>& n, 
 // The rest of the tube detector for a located packet: the first of the candidate tubes the
 // ray enters, the absorption point drawn from the truncated exponential of the 3He path
 // (u_det), pixel, time of flight and bin.
-template <typename R, bool NORM = false, int FORM = 0>
+template <typename R, bool SWAP = false, bool QUOTIENT = false>
 __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W,
                                                const R* __restrict__ tu, const Ray<R>& n,
                                                R u_det, int row, int g) {
@@ -1542,7 +1537,7 @@ __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W
     const int c = g + dc;
     if (c < 0 || c >= n_tubes_row) continue;
     R s1, s2;
-    if (!tube_span<R, NORM, FORM>(Rad, tu[2 * c], tu[2 * c + 1], (R)D.tube_r, n, &s1, &s2)) continue;
+    if (!tube_span<R, SWAP, QUOTIENT>(Rad, tu[2 * c], tu[2 * c + 1], (R)D.tube_r, n, &s1, &s2)) continue;
     R ys1, ys2;
     if (M::is_zero(n.dy)) {
       if (!(n.y >= y_lo && n.y <= y_hi)) continue;
@@ -1584,12 +1579,12 @@ __device__ __forceinline__ Hit<R> tubes_absorb(const DetP<R>& D, const TofWin& W
 // Tube detector system (section 2.4.3, "Ray tracing in a detector system"): the packet's
 // crossing of the tube-centre circle picks the row and three candidate tubes; the first
 // tube the ray enters absorbs it.
-template <typename R, bool NORM, int FORM>
+template <typename R, bool SWAP, bool QUOTIENT>
 __device__ __forceinline__ Hit<R> detect_tubes(const DetP<R>& D, const TofWin& W,
                                                const R* __restrict__ tu, const Ray<R>& n,
                                                R u_det) {
   int row = 0, g = 0;
-  if (!tubes_locate<R, NORM>(D, n, &row, &g)) {
+  if (!tubes_locate<R, SWAP>(D, n, &row, &g)) {
     Hit<R> h;
     h.bin = -1;
     h.pixel = -1;
@@ -1598,22 +1593,25 @@ __device__ __forceinline__ Hit<R> detect_tubes(const DetP<R>& D, const TofWin& W
     h.pabs = R(0);
     return h;
   }
-  return tubes_absorb<R, NORM, FORM>(D, W, tu, n, u_det, row, g);
+  return tubes_absorb<R, SWAP, QUOTIENT>(D, W, tu, n, u_det, row, g);
 }
 
-// FP32 rounding of the detector trace.  The compiler's choice of fused multiply-adds differs from
-// kernel to kernel and with the code around; where a kernel's packets are detected in the same
-// block they are loaded in, it would have changed the detected weights of grazing chords by up
-// to 1e-4 of themselves.  The two expressions concerned are therefore written out:
-// NORM: the direction's squared horizontal length, fma(dz, dz, dx dx) (Mth::norm2);
-// FORM: r^2 - cr^2/a of a tube's chord, 1: fma(r, r, -(cr^2/a)), 2: fma(-cr^2, 1/a, r^2), 0: as the
-// compiler has it.
-template <typename R, int DET, bool NORM = false, int FORM = 0, class Rng>
+// FP32 rounding of the detector trace.  A chord next to the tube's edge, r^2 - d^2 of two nearly
+// equal numbers, is its rounding, and the compiler's choice of fused multiply-adds differs with
+// the code around.  The expressions concerned are therefore written out:
+//   a, the direction's squared horizontal length: fma(dz, dz, dx dx) (Mth::norm2); SWAP: with dx and
+//   dz exchanged (stored packets);
+//   r^2 - cr^2/a of a tube's chord: fma(-cr^2, 1/a, r^2); QUOTIENT: fma(r, r, -(cr^2/a)) (batched
+//   launches, and single ones of one-scatterer powder samples).
+// Each is within 2^-22 r^2 of the exact value.  Between the two chords 0.15 % of a histogram's bins
+// differ, by 1e-7 to 2e-6 of the histogram; one of them in all kernels would move the FP32 results
+// of the others by that much.
+template <typename R, int DET, bool SWAP = false, bool QUOTIENT = false, class Rng>
 __device__ __forceinline__ Hit<R> detect(const DetP<R>& D, const TofWin& W, const R* tu,
                                          const Rng& rng, int order, const Ray<R>& n) {
-  if (DET == MCV_DET_SURFACE) return detect_surface<R, NORM>(D, W, n);
+  if (DET == MCV_DET_SURFACE) return detect_surface<R, SWAP>(D, W, n);
   const R u = rng.template first<R>(order, 3);
-  return detect_tubes<R, NORM, FORM>(D, W, tu, n, u);
+  return detect_tubes<R, SWAP, QUOTIENT>(D, W, tu, n, u);
 }
 
 // ---- tallies ---------------------------------------------------------------------------

@@ -535,8 +535,8 @@ struct LaneMisses {
 
 // The waves of one warp over neutron ids first_id + [lo, hi) of one simulation, and over
 // every further range `src` hands out for it.  Returns with both queues empty.
-// FORM: see detect().
-template <typename R, int NS, int DET, int KS, int FORM, class Job, class Src, class P>
+// QUOTIENT: see detect().
+template <typename R, int NS, int DET, int KS, bool QUOTIENT, class Job, class Src, class P>
 __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, int64_t lo,
                                           int64_t hi, const R* tu, P& pol, Src& src) {
   const SampleP<R>& S = job.S();
@@ -650,8 +650,10 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
       h.pixel = -1;
       h.w_det = R(0);
       // The wide kernels load the packets in a block of their own: the compiler's choice of
-      // fused multiply-adds depends on the block, and the FP32 results on that choice.  (In
-      // one block, as the powder kernels have it, fewer registers spill: 4.93 -> 4.66 ms.)
+      // fused multiply-adds depends on the block, and the FP32 results on that choice.  In one
+      // block, as the powder kernels have it, fewer registers spill (vanadium-like, 1e7: 1328 ->
+      // 1309 us; 13 crystal orientations: 4119 -> 3949 us), but the single crystal's histograms
+      // move by 7e-6 of themselves.
       Ray<R> pe;
       int order = 0, row = 0, g = 0;
       int64_t nid = 0;
@@ -679,7 +681,7 @@ __device__ __forceinline__ void run_waves(const TraceArgs& A, const Job& job, in
         if constexpr (kLocateEarly)
           h = tubes_absorb<R>(D, job.W(), tu, pe, rng.template first<R>(order, 3), row, g);
         else
-          h = detect<R, DET, KS == kKernelsPowder, FORM>(D, job.W(), tu, rng, order, pe);
+          h = detect<R, DET, false, QUOTIENT>(D, job.W(), tu, rng, order, pe);
       }
       __syncwarp();
       pol.record(A, have, h);
@@ -710,7 +712,7 @@ __global__ void __launch_bounds__(WaveCfg<R>::threads, 1)
   const int64_t lo = (A.n * wid) / nw, hi = (A.n * (wid + 1)) / nw;
   NoMoreIds src;
   const ParamJob<R> job{A};
-  run_waves<R, NS, DET, KS, NS == 1 && KS == kKernelsPowder ? 1 : 2>(A, job, lo, hi, tu, pol, src);
+  run_waves<R, NS, DET, KS, NS == 1 && KS == kKernelsPowder>(A, job, lo, hi, tu, pol, src);
   pol.flush(A, threadIdx.x & 31);
 }
 
@@ -722,7 +724,7 @@ __global__ void __launch_bounds__(WaveCfg<R>::threads, 1)
 // block into its slot of shared memory, and keeps taking items of it -- without draining its
 // queues between items -- until that queue is empty; then it moves on to the next
 // simulation that still has items.  Each neutron's arithmetic is the single-simulation
-// kernel's.
+// kernel's (in FP32 up to the last bits: detect()).
 // SS: every simulation has the batch's sample (A.Sf / A.Sd), kept in parameter space
 template <typename R, int NS, int DET, int KS, bool SS, bool EV>
 __global__ void __launch_bounds__(WaveCfg<R>::threads, 1)
@@ -775,7 +777,7 @@ __global__ void __launch_bounds__(WaveCfg<R>::threads, 1)
     uint32_t* to = reinterpret_cast<uint32_t*>(&me.sim);
     for (int w = lane; w < (int)(sizeof(SimP<R>) / 4); w += 32) to[w] = from[w];
     __syncwarp();
-    run_waves<R, NS, DET, KS, 1>(A, job, lo, hi, tu, pol, src);
+    run_waves<R, NS, DET, KS, true>(A, job, lo, hi, tu, pol, src);
     pol.flush(A, lane);
   }
 }
@@ -817,7 +819,7 @@ __device__ __forceinline__ void detect_slot(const TraceArgs& A, const EventsArgs
   if (!load_input<R>(A, i, &n)) return;
   cnt.nemit++;
   const NeutronRng rng(A.keys, A.in_id[i]);
-  const Hit<R> h = detect<R, DET>(Dof<R>(A), Dof<R>(A).win, tu, rng, o, n);
+  const Hit<R> h = detect<R, DET, true>(Dof<R>(A), Dof<R>(A).win, tu, rng, o, n);
   if (h.pixel >= 0 && A.ev.count) append_event(A.ev, h.pixel, h.tof.value(), (double)h.w_det);
   if (h.bin >= 0) {
     if (h.bin >= Dof<R>(A).n_bins) {
