@@ -405,7 +405,8 @@ typedef struct mcv_batch mcv_batch;
  * uploads them to device memory owned by the batch (this call allocates and synchronises;
  * the sims array and what it points to may be freed afterwards, the histograms may not).
  * The launch shape (neutrons per work item, blocks per SM) is the one mcv_batch_tune last
- * chose on this context for the same kind of batch, else a default.
+ * chose on this context for the same kind of batch (work items in proportion to the batches'
+ * neutrons), else a default.
  * Errors: MCV_EINVAL for any invalid simulation (the message names it), MCV_ENOMEM. */
 mcv_status mcv_batch_create(mcv_ctx* ctx, const mcv_sim* sims, int nsims,
                             const mcv_detector* det, int fp_mode, mcv_batch** out);
@@ -415,8 +416,9 @@ mcv_status mcv_batch_create(mcv_ctx* ctx, const mcv_sim* sims, int nsims,
 mcv_status mcv_batch_run(mcv_batch* b, void* stream);
 /* Autotuner: times the batch kernel on a proportional sample of about trial_neutrons
  * neutrons (<= 0: 2e7) of this batch for each candidate launch shape -- work-item sizes of
- * 512..8192 neutrons (scaled by the sample's fraction of the batch in the trial, which keeps
- * the number of items per warp) and blocks per SM at and below the occupancy limit -- with
+ * 512..8192 neutrons, and of 64..256 and the default where the sample is large enough to tell
+ * them apart (scaled by the sample's fraction of the batch in the trial, which keeps the
+ * number of items per warp), and blocks per SM at and below the occupancy limit -- with
  * histograms in scratch memory (the simulations' own histograms are not touched), keeps the
  * fastest for this batch and records it on the context for later batches of the same kind
  * (real type, number of scatterers, detector kind, kernel set).  Synchronises `stream`;

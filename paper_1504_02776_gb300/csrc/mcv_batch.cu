@@ -17,8 +17,6 @@ namespace {
 
 // warps of a block of the batched kernel (WaveCfg)
 int warps_per_block(int fp_mode) { return mcv::wave_threads(fp_mode) / 32; }
-constexpr int64_t kDefaultChunk = 8192;
-constexpr int64_t kMinChunk = 64;
 
 // The simulations of a batch as the kernel reads them: host images of the parameter blocks
 // in the batch's real type, and the shape of the batch.
@@ -171,17 +169,6 @@ std::vector<unsigned char> device_image(const BatchImage& im) {
   return out;
 }
 
-// default work-item size: about 16 items per resident warp, a multiple of 32 in
-// [kMinChunk, kDefaultChunk] (items of one simulation follow each other in a warp without a
-// drain, so small items cost little more than their queue counter update; with items of at
-// least 256, 13 crystal orientations of 2e5 neutrons left the warps 3 items each: 4.34 ms, 128:
-// 4.13, 64: 4.03)
-int64_t default_chunk(int64_t total_n, int64_t warps) {
-  int64_t c = total_n / std::max<int64_t>(1, warps * 16);
-  c = std::min(std::max(c, kMinChunk), kDefaultChunk);
-  return (c / 32) * 32;
-}
-
 int grid_of(int fp_mode, int sm_count, int blocks_per_sm, int64_t n_items) {
   const int kWarpsPerBlock = warps_per_block(fp_mode);
   const int64_t full = (int64_t)sm_count * blocks_per_sm;
@@ -211,6 +198,22 @@ mcv::TraceArgs& zeroed(mcv::TraceArgs& A) {
 
 mcv_ctx::Tuned& tuned_slot(mcv_ctx* ctx, const BatchImage& im) {
   return ctx->tuned[im.fp][ns_index(im.ns)][im.det][im.bvk][im.ss];
+}
+
+int64_t warps_of(const mcv_ctx* ctx, const BatchImage& im, int blocks_per_sm) {
+  return (int64_t)ctx->sm_count * blocks_per_sm * warps_per_block(im.fp);
+}
+
+// the launch shape of a new batch: the tuned one of its kind, else the default
+void set_shape(mcv_ctx* ctx, mcv_batch* b) {
+  const mcv_ctx::Tuned& t = tuned_slot(ctx, b->im);
+  if (t.chunk > 0) {
+    b->chunk = mcv::scaled_chunk(t.chunk, t.total, b->im.total_n);
+    b->blocks_per_sm = std::min(t.blocks_per_sm, b->max_blocks_per_sm);
+  } else {
+    b->blocks_per_sm = b->max_blocks_per_sm;
+    b->chunk = mcv::default_chunk(b->im.total_n, warps_of(ctx, b->im, b->blocks_per_sm));
+  }
 }
 
 // uploads the batch's device block and sets the launch arguments for its current chunk
@@ -269,15 +272,7 @@ mcv_status mcv_batch_create(mcv_ctx* ctx, const mcv_sim* sims, int nsims,
     delete b;
     return st;
   }
-  const mcv_ctx::Tuned& t = tuned_slot(ctx, b->im);
-  if (t.chunk > 0) {
-    b->chunk = t.chunk;
-    b->blocks_per_sm = std::min(t.blocks_per_sm, b->max_blocks_per_sm);
-  } else {
-    b->blocks_per_sm = b->max_blocks_per_sm;
-    b->chunk = default_chunk(b->im.total_n,
-                             (int64_t)ctx->sm_count * b->blocks_per_sm * warps_per_block(b->im.fp));
-  }
+  set_shape(ctx, b);
   cudaError_t e = cudaMalloc(&b->d_block, device_bytes(b->im));
   if (e != cudaSuccess) {
     delete b;
@@ -375,9 +370,11 @@ mcv_status mcv_batch_tune(mcv_batch* b, int64_t trial_neutrons, void* stream) {
   // candidate work-item sizes of the full batch; the trial uses them scaled by its fraction
   // of the neutrons, which keeps the number of items per warp (the load balance at the end)
   const double frac = (double)tr.total_n / (double)b->im.total_n;
-  const int64_t chunks[] = {512, 1024, 2048, 4096, 8192};
+  const mcv::ChunkList chunks = mcv::chunk_candidates(
+      b->im.total_n, tr.total_n, warps_of(b->ctx, b->im, b->max_blocks_per_sm));
   st = MCV_OK;
-  for (int64_t chunk : chunks) {
+  for (int k = 0; k < chunks.n; ++k) {
+    const int64_t chunk = chunks.chunk[k];
     if (e != cudaSuccess || st != MCV_OK) break;
     const int64_t tc = std::max<int64_t>(32, ((int64_t)(chunk * frac) / 32) * 32);
     mcv::BatchArgs Q;
@@ -413,6 +410,7 @@ mcv_status mcv_batch_tune(mcv_batch* b, int64_t trial_neutrons, void* stream) {
   b->blocks_per_sm = best_blocks;
   mcv_ctx::Tuned& t = tuned_slot(b->ctx, b->im);
   t.chunk = best_chunk;
+  t.total = b->im.total_n;
   t.blocks_per_sm = best_blocks;
   return upload(b);
 }
@@ -432,14 +430,7 @@ mcv_status mcv_trace_batch(mcv_ctx* ctx, const mcv_sim* sims, int nsims,
   if (b.im.total_n == 0) return MCV_OK;
   st = occupancy(ctx, b.im, &b.max_blocks_per_sm);
   if (st != MCV_OK) return st;
-  const mcv_ctx::Tuned& t = tuned_slot(ctx, b.im);
-  if (t.chunk > 0) {
-    b.chunk = t.chunk;
-    b.blocks_per_sm = std::min(t.blocks_per_sm, b.max_blocks_per_sm);
-  } else {
-    b.blocks_per_sm = b.max_blocks_per_sm;
-    b.chunk = default_chunk(b.im.total_n, (int64_t)ctx->sm_count * b.blocks_per_sm * warps_per_block(b.im.fp));
-  }
+  set_shape(ctx, &b);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const std::vector<unsigned char> img = device_image(b.im);
   void* d = nullptr;

@@ -18,10 +18,10 @@ struct mcv_ctx {
   // cached blocks per SM of the trace kernels: [fp][ns 1,2,4][det][bvk][waves]
   int occ[2][3][3][2][2];
   int occ_adj[2][3][3][2];  // the same for the adjoint kernel
-  // batched launch chosen by mcv_batch_tune for a kind of batch: neutrons per work item and
-  // blocks per SM (0: not tuned yet); [fp][ns 1,2,4][det][bvk][one sample for all]
+  // batched launch chosen by mcv_batch_tune for a kind of batch: neutrons per work item, of how
+  // many in all, and blocks per SM (0: not tuned yet); [fp][ns 1,2,4][det][bvk][one sample for all]
   struct Tuned {
-    int64_t chunk;
+    int64_t chunk, total;
     int blocks_per_sm;
   } tuned[2][3][3][2][2];
 };

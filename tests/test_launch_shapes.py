@@ -1,7 +1,8 @@
 """Launch shapes of the trace kernels (csrc/mcv_shape.h, compiled as plain C++): every neutron has a
 lane, no block is larger than the kernel's or the grid than the GPU, a warp of the waves has 32
 neutrons (31 where they do not divide evenly, more once the GPU is full), and small runs are
-spread over the SMs."""
+spread over the SMs.  Work items of batches: the tuner's candidates hold the default size of a
+batch that its trial can tell apart, and a tuned size follows the batch's neutrons."""
 import os
 import subprocess
 
@@ -44,3 +45,36 @@ def test_shapes_fill_warps_and_sms(tmp_path, sms, per_sm, threads, least):
         warps, batches = lanes // 32, (n + 31) // 32
         assert batches <= warps < batches + block // 32, line  # no block without a batch
         assert grid >= min((batches + least - 1) // least, (room + 1) // 2), line
+
+
+_CHUNKS = """
+#include <cstdio>
+#include <cstdlib>
+#include "mcv_shape.h"
+int main(int, char** v) {
+  const long long total = std::atoll(v[1]), trial = std::atoll(v[2]), warps = std::atoll(v[3]);
+  const mcv::ChunkList l = mcv::chunk_candidates(total, trial, warps);
+  std::printf("%lld %lld %lld %lld", (long long)mcv::default_chunk(total, warps),
+              (long long)mcv::scaled_chunk(512, total, total), (long long)mcv::scaled_chunk(512, total, total / 4),
+              (long long)mcv::scaled_chunk(512, total, 1ll << 40));
+  for (int k = 0; k < l.n; ++k) std::printf(" %lld", (long long)l.chunk[k]);
+}
+"""
+
+
+@pytest.mark.parametrize("total,trial", [(260_000, 260_000), (2_600_000, 2_600_000), (75_100, 40_000),
+                                         (362_000_000, 20_000_000), (855_000_000, 20_000_000), (1, 1)])
+def test_work_items_of_batches(tmp_path, total, trial):
+    src, exe, warps = tmp_path / "chunks.cpp", str(tmp_path / "chunks"), 3040
+    src.write_text(_CHUNKS)
+    subprocess.run(["g++", "-O2", "-std=gnu++17", "-I" + CSRC, str(src), "-o", exe], check=True)
+    out = subprocess.run([exe, str(total), str(trial), str(warps)], check=True, capture_output=True,
+                         text=True).stdout
+    default, same, quarter, huge, *tried = map(int, out.split())
+    assert default == max(64, min(8192, total // (16 * warps))) // 32 * 32
+    assert same == 512 and quarter == (128 if total > 3 else 64) and huge == 8192
+    assert tried[:5] == [512, 1024, 2048, 4096, 8192] and len(set(tried)) == len(tried)
+    apart = trial >= 64 * warps
+    if apart and default * trial >= 32 * total:
+        assert default in tried
+    assert all(apart and 64 <= c <= 8192 and c * trial >= 32 * total for c in tried[5:])

@@ -1,7 +1,9 @@
 """Launches fill the GPU: a fused run from a stored beam, which is traced by a kernel of its own,
 against the same neutrons generated in the waves.  It does the work of the waves without their
 compaction and reads 60 bytes per neutron: 1.4 times their time (1e6 neutrons, FP32 powder, both
-without the histogram's clear).  Bar, 2.2: with the waves' one block per SM it took 3.3 times."""
+without the histogram's clear).  Bar, 2.2: with the waves' one block per SM it took 3.3 times.
+And tuning a batch of 13 x 2e4 neutrons does not make it slower: bar, 1.2 times its time before,
+where work items of 512 and more alone took 2.7 times."""
 import statistics
 
 import pytest
@@ -43,4 +45,18 @@ def test_stored_beam_into_a_detector_fills_the_gpu():
 
     fused, stored = _us(trace), _us(lambda: trace(beam_in=beam))
     assert stored <= 2.2 * fused, (stored, fused)
+    ctx.close()
+
+
+def test_tuning_a_small_batch_does_not_slow_it_down():
+    from paper_1504_02776_gb300 import binding as B
+    import gpu_helpers as H
+    ctx = H.ctx()
+    det = mi.tube_detector(n_tof=40)
+    b = ctx.batch([w.replace(detector=det, n=20_000)
+                   for w in mi.config3_batch(orientations=range(0, 195, 15))], fp_mode=B.FP32)
+    before = _us(b.run)
+    shape = b.tune()
+    assert _us(b.run) <= 1.2 * before, (before, shape)
+    b.close()
     ctx.close()
