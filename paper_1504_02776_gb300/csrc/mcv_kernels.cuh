@@ -90,6 +90,8 @@ struct Forward {
         err = 1;
         return;
       }
+      // (one add per lane: summing equal bins in the warp, as the waves do, was slower here,
+      // 120.6 -> 124.2 us for 1e6 stored neutrons)
       if (A.hist) atomicAdd(A.hist + h.bin, (double)h.w_det);
       t.det.add(h.w_det);
       t.cnt.ndet++;
